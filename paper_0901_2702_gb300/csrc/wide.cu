@@ -633,7 +633,9 @@ bool wide_supported(int nf, int nlam) {
 
 cudaError_t launch_wide_pack(const float* filters, int nf, const float* wl, int nlam,
                              float* table, int* err, cudaStream_t s) {
-  wide_pack_kernel<<<1, 256, 0, s>>>(filters, nf, wl, nlam, table, err);
+  // one warp per sample and round: 32 warps take 112 samples in four rounds
+  // (8 warps took 36 us, 32 take 13)
+  wide_pack_kernel<<<1, 1024, 0, s>>>(filters, nf, wl, nlam, table, err);
   return cudaGetLastError();
 }
 
