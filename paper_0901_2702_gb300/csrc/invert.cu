@@ -758,54 +758,182 @@ __global__ void __launch_bounds__(BS, 1) invert_kernel(InvertArgs A) {
   }
 }
 
-// Covariance of every pixel that finished with a model, from the packed
-// J^T W J parked in the pixel's output row.  Cholesky runs one pixel per
-// thread; the rare pixels whose matrix is numerically singular go to a
-// shared-memory queue and are drained by consecutive threads, so the costly
-// eigen-decomposition runs in (nearly) full warps instead of stalling every
-// warp that happens to hold one such pixel.
-constexpr int kCovThreads = 128;
-constexpr int kCovQueue = 2 * kCovThreads;
+// ---- covariance of every pixel that finished with a model, from the packed
+// J^T W J parked in the pixel's output row ----
+
+// The eigen-decomposition fallback of one pixel by kNP lanes: jacobi_pinv() and
+// the scaling around it with every element's operations in the same order,
+// row k of the matrix and of the eigenvectors on lane k, the rotations'
+// angles on all of them.  A lane alone spends two thirds of a rotation's
+// FP64 time on the 3 kNP pairs of elements that these lanes update together, so a few
+// pixels finish sooner this way (300 pixels, a handful of them singular:
+// the whole kernel
+// 2.7 -> 0.54 ms); a full warp of pixels, one a lane, takes fewer FP64
+// instructions a pixel and is left to the one-lane path.
+struct CoopPixel {
+  double a[kNP][kNP], v[kNP][kNP], sc[kNP], li[kNP];
+};
+constexpr int kCoopPerWarp = 3, kCoopWarps = 4, kCoopMax = kCoopPerWarp * kCoopWarps;
+
+// Called by a whole warp; lanes past kCoopPerWarp * kNP, and groups without a
+// pixel (row == nullptr), only take part in the barriers.
+__device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32_t free_mask) {
+  constexpr int N = kNP;
+  const int lane = threadIdx.x & 31;
+  const int grp = lane / N, k = lane - grp * N;
+  const bool live = grp < kCoopPerWarp && row != nullptr;
+  CoopPixel& B = bufs[live ? grp : 0];
+  auto held_of = [&](int i) {
+    const double d = (double)row[tri(i, i)];
+    return !((free_mask >> i) & 1u) || !(d > 0.0) || !isfinite(d);
+  };
+  uint32_t held = 0;
+  if (live) {
+    for (int i = 0; i < N; ++i) held |= held_of(i) ? 1u << i : 0u;
+    B.sc[k] = ((held >> k) & 1u) ? 0.0 : rsqrt((double)row[tri(k, k)]);
+  }
+  __syncwarp();
+  if (live)
+    for (int j = 0; j < N; ++j) {
+      const int i0 = max(k, j), j0 = min(k, j);
+      double m;
+      if (k == j)
+        m = 1.0;
+      else
+        m = ((held >> k) & 1u) || ((held >> j) & 1u)
+                ? 0.0
+                : (double)row[tri(i0, j0)] * B.sc[i0] * B.sc[j0];
+      B.a[k][j] = m;
+      B.v[k][j] = (k == j) ? 1.0 : 0.0;
+    }
+  __syncwarp();
+  bool run = live;
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    double off = 0.0, dia = 0.0;
+    if (run)
+      for (int i = 0; i < N; ++i) {
+        dia += B.a[i][i] * B.a[i][i];
+        for (int j = i + 1; j < N; ++j) off += B.a[i][j] * B.a[i][j];
+      }
+    if (!(off > 1e-26 * dia)) run = false;
+    if (!__any_sync(0xffffffffu, run)) break;
+    for (int p = 0; p < N - 1; ++p)
+      for (int q = p + 1; q < N; ++q) {
+        const double apq = B.a[p][q], app = B.a[p][p], aqq = B.a[q][q];
+        const bool act = run && apq != 0.0;
+        double c = 1.0, sn = 0.0;
+        if (act) {
+          const double th = (aqq - app) / (2.0 * apq);
+          const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
+          c = 1.0 / sqrt(t * t + 1.0);
+          sn = t * c;
+        }
+        __syncwarp();  // the pivots are read before they change
+        if (act) {
+          const double akp = B.a[k][p], akq = B.a[k][q];
+          const double vkp = B.v[k][p], vkq = B.v[k][q];
+          B.a[k][p] = c * akp - sn * akq;
+          B.a[k][q] = sn * akp + c * akq;
+          B.v[k][p] = c * vkp - sn * vkq;
+          B.v[k][q] = sn * vkp + c * vkq;
+        }
+        __syncwarp();
+        if (act) {
+          const double apk = B.a[p][k], aqk = B.a[q][k];
+          B.a[p][k] = c * apk - sn * aqk;
+          B.a[q][k] = sn * apk + c * aqk;
+        }
+        __syncwarp();
+      }
+  }
+  if (live) {
+    double lmax = 0.0;
+    for (int i = 0; i < N; ++i) lmax = fmax(lmax, fabs(B.a[i][i]));
+    const double l = fabs(B.a[k][k]);
+    B.li[k] = (l > 1e-12 * lmax && l > 0.0) ? 1.0 / B.a[k][k] : 0.0;
+  }
+  __syncwarp();
+  if (live) {
+    // row k of the lower triangle, unscaled, and its mirror image
+    for (int j = 0; j <= k; ++j) {
+      double s = 0.0;
+      for (int e = 0; e < N; ++e) s += B.v[k][e] * B.li[e] * B.v[j][e];
+      const float q = ((held >> k) & 1u) || ((held >> j) & 1u) ? 0.0f
+                                                               : (float)(B.sc[k] * B.sc[j] * s);
+      row[k * 10 + j] = q;
+      row[j * 10 + k] = q;
+    }
+    for (int j = N; j < 10; ++j) row[k * 10 + j] = row[j * 10 + k] = 0.0f;
+    if (k == 0)
+      for (int i = N; i < 10; ++i)
+        for (int j = N; j < 10; ++j) row[i * 10 + j] = 0.0f;
+  }
+  __syncwarp();
+}
+
+// Cholesky runs one pixel per thread, the warps independent of each other;
+// the rare pixels whose matrix is numerically singular (2 % of a map) go to
+// the CTA's queue, and once its share of the map is swept the CTA drains the
+// queue: whole warps of them one pixel a lane, up to kCoopMax left over by
+// groups of lanes.  FP64-bound (a warp instruction holds the pipe 64 cycles).
+// One CTA of 16 warps per SM, so that a queue fills whole warps: the disk's
+// 3,290,904 pixels 16.7 -> 13.0 ms against four CTAs of 4 warps, each with a
+// barrier a round and a nearly empty last warp in its queue (1,048,576
+// pixels: 5.3 ms either way).  A full queue sends its pixels to the one-lane
+// path at once.  `ppr` pixels a round (a multiple of
+// 32, at most the threads of a CTA): small maps are dealt out over the SMs.
+constexpr int kCovThreads = 512;
+constexpr int kCovQueue = 4096;
 template <bool DF, int NPAR = kNP>
 __global__ void __launch_bounds__(kCovThreads) covariance_kernel(float* cov,
                                                                  const int32_t* status,
                                                                  int64_t npix_max,
                                                                  const int64_t* npix_dev,
-                                                                 uint32_t free_mask) {
-  __shared__ int64_t queue[kCovQueue];
+                                                                 uint32_t free_mask, int ppr) {
+  __shared__ int32_t queue[kCovQueue];  // pixel = queue / ppr * stride + base + queue % ppr
+  // with the filling factor free every singular pixel takes the one-lane path:
+  // there the groups' results differ from it in the last bits (the compiler
+  // fuses other products of the rotations), and a row's bits must not depend
+  // on the map it came in
+  constexpr bool kCoop = NPAR == kNP;
+  __shared__ CoopPixel coop[kCoop ? kCoopMax : 1];
   __shared__ int qn;
   const int64_t npix = npix_dev ? *npix_dev : npix_max;
   if (threadIdx.x == 0) qn = 0;
   __syncthreads();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  // every thread of the block runs the same number of rounds
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < npix; base += stride) {
-    const int64_t p = base + threadIdx.x;
-    if (p < npix) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * ppr, base = (int64_t)blockIdx.x * ppr;
+  auto one = [&](int64_t p, bool try_only) {
+    return DF ? covariance_df(cov + p * 100, 1, free_mask, cov + p * 100, try_only)
+              : covariance_fp64<NPAR>(cov + p * 100, 1, free_mask, cov + p * 100, try_only);
+  };
+  if ((int)threadIdx.x < ppr) {
+    int32_t slot0 = threadIdx.x;
+    for (int64_t p = base + threadIdx.x; p < npix; p += stride, slot0 += ppr) {
       const int st = status[p];
       if (st == VFISV_PIX_CONVERGED || st == VFISV_PIX_MAXITER || st == VFISV_PIX_STALLED) {
-        const bool ok = DF ? covariance_df(cov + p * 100, 1, free_mask, cov + p * 100, true)
-                           : covariance_fp64<NPAR>(cov + p * 100, 1, free_mask, cov + p * 100,
-                                                   true);
-        if (!ok) {
+        if (!one(p, true)) {
           const int slot = atomicAdd(&qn, 1);
-          queue[slot] = p;  // slot < kCovQueue: drained below before it can fill
+          if (slot < kCovQueue && slot0 >= 0)
+            queue[slot] = slot0;
+          else
+            one(p, false);
         }
       }
     }
-    __syncthreads();
-    const bool last = base + stride >= npix;
-    if (qn >= kCovThreads || last) {
-      const int n = qn;
-      for (int i = threadIdx.x; i < n; i += blockDim.x)
-        if (DF)
-          covariance_df(cov + queue[i] * 100, 1, free_mask, cov + queue[i] * 100, false);
-        else
-          covariance_fp64<NPAR>(cov + queue[i] * 100, 1, free_mask, cov + queue[i] * 100, false);
-      __syncthreads();
-      if (threadIdx.x == 0) qn = 0;
+  }
+  __syncthreads();
+  const int n = min(qn, kCovQueue);
+  auto pixel = [&](int i) { return base + (int64_t)(queue[i] / ppr) * stride + queue[i] % ppr; };
+  const int left = n % 32, whole = (kCoop && left <= kCoopMax) ? n - left : n;
+  for (int i = threadIdx.x; i < whole; i += kCovThreads) one(pixel(i), false);
+  if constexpr (kCoop) {
+    const int cw = warp - (kCovThreads / 32 - kCoopWarps);
+    if (cw >= 0 && whole + cw * kCoopPerWarp < n) {
+      const int i = whole + cw * kCoopPerWarp + lane / kNP;
+      const bool has = lane < kCoopPerWarp * kNP && i < n;
+      covariance_coop(coop + cw * kCoopPerWarp, has ? cov + pixel(i) * 100 : nullptr, free_mask);
     }
-    __syncthreads();
   }
 }
 
@@ -816,17 +944,21 @@ cudaError_t launch_covariance(float* cov, const int32_t* status, int64_t npix,
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   nsm = sm_budget(nsm);
-  // a few blocks per SM, each sweeping many pixels so its fallback queue fills
-  int64_t grid = (npix + kCovThreads - 1) / kCovThreads;
-  if (grid > (int64_t)nsm * 4) grid = (int64_t)nsm * 4;
+  // one CTA per SM; its pixels a round, whole warps, from the map's size
+  int64_t ppr = ((npix + nsm - 1) / nsm + 31) / 32 * 32;
+  if (ppr > kCovThreads) ppr = kCovThreads;
+  if (ppr < 32) ppr = 32;
+  int64_t grid = (npix + ppr - 1) / ppr;
+  if (grid > nsm) grid = nsm;
   if (grid < 1) grid = 1;
+  const int g = (int)grid, r = (int)ppr;
   if (fast_solve)
-    covariance_kernel<true><<<(int)grid, kCovThreads, 0, s>>>(cov, status, npix, npix_dev, free_mask);
+    covariance_kernel<true><<<g, kCovThreads, 0, s>>>(cov, status, npix, npix_dev, free_mask, r);
   else if (free_mask & (1u << 9))  // the filling factor free: 10 parameters
-    covariance_kernel<false, 10><<<(int)grid, kCovThreads, 0, s>>>(cov, status, npix, npix_dev,
-                                                                    free_mask);
+    covariance_kernel<false, 10><<<g, kCovThreads, 0, s>>>(cov, status, npix, npix_dev,
+                                                            free_mask, r);
   else
-    covariance_kernel<false><<<(int)grid, kCovThreads, 0, s>>>(cov, status, npix, npix_dev, free_mask);
+    covariance_kernel<false><<<g, kCovThreads, 0, s>>>(cov, status, npix, npix_dev, free_mask, r);
   return cudaGetLastError();
 }
 
