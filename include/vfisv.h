@@ -296,8 +296,11 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
 
 /* Set the launch shape of the handle's filter-position LM kernel directly:
  * block in {64, 128, 256} threads per CTA with tpp in {1, 2, 4} threads per
- * pixel, or block = 384 with tpp = 1 for the warp-specialised kernel
- * (default 128 x 1).  VFISV_E_ARG for any other value. */
+ * pixel, or block = 384 with tpp = 1 for the warp-specialised kernel.  Until a
+ * shape is set (here or by vfisv_autotune) the library chooses by the size of
+ * the map: a kernel with eight lanes per pixel for maps of up to a few tens of
+ * thousands of pixels, the warp-specialised one above; results are the same
+ * bits as with 128 x 1.  VFISV_E_ARG for any other value. */
 int vfisv_set_launch_shape(vfisv_handle* h, int32_t block, int32_t tpp);
 
 /* Persistent launches of this handle (the LM, wide, covariance and network

@@ -27,7 +27,7 @@ struct vfisv_handle {
   size_t nnws_bytes = 0;
   void* mixws = nullptr;   // mixed inversion: guesses, gathered pixels, 2nd run
   size_t mixws_bytes = 0;
-  int lm_block = 128;      // LM threads per CTA (vfisv_autotune)
+  int lm_block = 0;        // LM threads per CTA (vfisv_autotune; 0: by the map's size)
   int lm_tpp = 1;          // LM threads per pixel (vfisv_autotune)
   void* vtab = nullptr;    // Taylor table of H, F (built on first use)
   void* geom = nullptr;    // filter centres and wing weights of the weak-field init

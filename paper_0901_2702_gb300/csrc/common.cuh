@@ -248,6 +248,13 @@ constexpr int kInvWsBlock = 384;
 cudaError_t invert_ws_set_constants(const Weideman& W);
 cudaError_t invert_ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem);
 cudaError_t launch_invert_ws(const InvertArgs& a, int grid, size_t smem, cudaStream_t s);
+// The kernel for maps too small to fill the chip one pixel a thread
+// (invert_lanes.cu): kInvLanes lanes a pixel, CTAs of kInvLanesBlock threads
+// (one warp); the same configuration.
+constexpr int kInvLanes = 8, kInvLanesBlock = 32;
+cudaError_t invert_lanes_set_constants(const Weideman& W);
+cudaError_t invert_lanes_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem);
+cudaError_t launch_invert_lanes(const InvertArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_covariance(float* cov, const int32_t* status, int64_t npix,
                               const int64_t* npix_dev, uint32_t free_mask, int fast_solve,
                               cudaStream_t s);

@@ -1026,10 +1026,30 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
     *tpp = 1;
     return slots_for<kInvThreadsDefault, false, false, true>(nlam, npix, nslots, grid, smem);
   }
-  if (*block == kInvWsBlock) {
-    if (!restarts && !fast_solve) {  // the warp-specialised kernel
+  const bool plain = !restarts && !fast_solve;
+  if (*block == 0) {
+    // no shape set: by the size of the map.  Up to twice the pixels that the
+    // kernel with several lanes a pixel holds at once (19,456 on 152 SMs) that
+    // kernel is the faster one -- 300 pixels 1.15 ms against 4.05 (128 x 1)
+    // and 5.35 (warp-specialised), 4,096 1.72 / 4.05 / 5.36, 12,288 3.46 /
+    // 4.07 / 5.33, 20,000 5.14 / 6.21 / 5.37 -- above it the warp-specialised
+    // one: 40,000 8.96 / 8.25 / 6.12, 1,048,576 204 / 138 / 101.
+    *block = kInvThreadsDefault;
+    if (plain) {
+      if (invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
+          npix <= 2 * *nslots)
+        *block = kInvLanesBlock;
+      else if (invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
+        *block = kInvWsBlock;
+      else
+        cudaGetLastError();
+    }
+  }
+  if (*block == kInvLanesBlock || *block == kInvWsBlock) {
+    if (plain) {
       *tpp = 1;
-      return invert_ws_slots(nlam, npix, nslots, grid, smem);
+      return *block == kInvWsBlock ? invert_ws_slots(nlam, npix, nslots, grid, smem)
+                                   : invert_lanes_slots(nlam, npix, nslots, grid, smem);
     }
     *block = kInvThreadsDefault;  // not compiled for this configuration
   }
@@ -1038,8 +1058,10 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
 }
 
 cudaError_t invert_set_constants(const Weideman& W) {
-  const cudaError_t e = cudaMemcpyToSymbol(c_W, &W, sizeof(W));
-  return e != cudaSuccess ? e : invert_ws_set_constants(W);
+  cudaError_t e = cudaMemcpyToSymbol(c_W, &W, sizeof(W));
+  if (e == cudaSuccess) e = invert_ws_set_constants(W);
+  if (e == cudaSuccess) e = invert_lanes_set_constants(W);
+  return e;
 }
 
 template <bool DF, int TPP>
@@ -1082,6 +1104,10 @@ cudaError_t launch_invert(const InvertArgs& a, int nf, int grid, int block, int 
   if (block == kInvWsBlock) {
     if (a.restarts || a.fast_solve || tpp != 1) return cudaErrorInvalidValue;
     return launch_invert_ws(a, grid, smem, s);
+  }
+  if (block == kInvLanesBlock) {
+    if (a.restarts || a.fast_solve || tpp != 1) return cudaErrorInvalidValue;
+    return launch_invert_lanes(a, grid, smem, s);
   }
   return a.fast_solve ? launch_invert_t<true>(a, grid, block, tpp, smem, s)
                       : launch_invert_t<false>(a, grid, block, tpp, smem, s);

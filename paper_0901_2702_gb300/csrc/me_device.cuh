@@ -19,11 +19,6 @@ constexpr int kWeidN = 16;
 #define VFISV_HORNER_UNROLL 15
 #endif
 constexpr int kHornerUnroll = VFISV_HORNER_UNROLL;
-// 1: multiply the filter weights by 1/Delta once per wavelength (6 products,
-// 6 live registers); 0: scale the six derivative row values instead.
-#ifndef VFISV_FOLD_ID_IN_WEIGHTS
-#define VFISV_FOLD_ID_IN_WEIGHTS 1
-#endif
 constexpr float kInvSqrtPi = 0.56418958354775628695f;
 constexpr float kTwoInvSqrtPi = 1.1283791670955125739f;
 constexpr float kDeg = 0.017453292519943295769f;
@@ -162,18 +157,18 @@ __device__ __forceinline__ RowScale row_scale(const LineK& lk, float eta0, float
 constexpr int kRows = 7;
 constexpr int kRowB = 1, kRowG = 2, kRowE = 3, kRowD = 4, kRowA = 5, kRowV = 6;
 
-// One wavelength point: synthesis (and, if DERIV, the Jacobian rows),
-// accumulated into acc[row][stokes][k] += T_k * value.
 // Rows of the non-magnetic (B = 0) Stokes I profile used when the filling
 // factor is free: value, then eta0 d/d eta0, u d/du, d/da, d/du (the scale
 // factors of the magnetic rows E, D, A, V apply to them alike).
 constexpr int kNmRows = 5;
 
-template <int NF, bool DERIV, bool NM = false>
-__device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, float x,
-                                            const float (&T)[NF],
-                                            float (&acc)[DERIV ? kRows : 1][4][NF],
-                                            float (*accn)[NF] = nullptr) {
+// The arithmetic of one wavelength point, handed out as it is formed: `out`
+// gets unit(yI, yQ, yU, yV), the unit-S1 Stokes values; with DERIV scale(iD),
+// the 1/Delta that every derivative row still lacks, then rows(S, vB, vG, vE,
+// vD, vA, vV) for each Stokes parameter S, and with NM the non-magnetic rows
+// nonmagnetic(v).
+template <bool DERIV, bool NM, class Out>
+__device__ __forceinline__ void lambda_point(const Weideman& W, const PixK& P, float x, Out& out) {
   const float up = fmaf(x, P.invD, -P.uv);
   const float ub = up + P.uB, ur = up - P.uB;
   float Hp, Fp, Hb, Fb, Hr, Fr;
@@ -203,13 +198,7 @@ __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, fl
   const float NU = eI * fmaf(eL, rV, -eV * rL);
   const float NV = fmaf(eI2, eV, rV * Pi);
   const float yI = NI * iD, yQ = -NQ * iD, yU = -NU * iD, yV = -NV * iD;
-#pragma unroll
-  for (int k = 0; k < NF; ++k) {
-    acc[0][0][k] = fmaf(T[k], yI, acc[0][0][k]);
-    acc[0][1][k] = fmaf(T[k], yQ, acc[0][1][k]);
-    acc[0][2][k] = fmaf(T[k], yU, acc[0][2][k]);
-    acc[0][3][k] = fmaf(T[k], yV, acc[0][3][k]);
-  }
+  out.unit(yI, yQ, yU, yV);
   if constexpr (DERIV) {
     // Eqs. 8-9: alpha = dH/da = -dF/du, beta = dH/du = dF/da
     const float a2 = 2.0f * P.a;
@@ -230,15 +219,7 @@ __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, fl
     const float gV = P.g2 * Hdif;
     const float gRL = P.g1 * fL;
     const float gRV = P.g2 * Fdif;
-#if VFISV_FOLD_ID_IN_WEIGHTS
-    // Weights of the derivative rows: the 1/Delta of every partial is folded
-    // into the filter weight.
-    float Td[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) Td[k] = T[k] * iD;
-#else
-    const float (&Td)[NF] = T;
-#endif
+    out.scale(iD);
 
     // For each Stokes parameter: the partials p_X = Delta * dy_S/dX w.r.t.
     // the five elements, then the chain rule through the profiles.
@@ -255,26 +236,14 @@ __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, fl
       const float Gp = fmaf(SHp, bep, -SFp * alp);
       const float Gb = fmaf(SHb, beb, -SFb * alb);
       const float Gr = fmaf(SHr, ber, -SFr * alr);
-      float vB = Gb - Gr;                                  // x kB
-      float vG = fmaf(peq, gIL, fmaf(pv, gV, fmaf(pr, gRL, pt * gRV)));
-      float vE = fmaf(pe, eI - 1.0f, fmaf(pq, eL, fmaf(pv, eV, fmaf(pr, rL, pt * rV))));
-      float vD = fmaf(up, Gp, fmaf(ub, Gb, ur * Gr));      // x (-1/dlambdaD)
-      float vA = fmaf(SHp, alp, fmaf(SFp, bep, fmaf(SHb, alb, fmaf(SFb, beb,
+      const float vB = Gb - Gr;                                  // x kB
+      const float vG = fmaf(peq, gIL, fmaf(pv, gV, fmaf(pr, gRL, pt * gRV)));
+      const float vE = fmaf(pe, eI - 1.0f, fmaf(pq, eL, fmaf(pv, eV, fmaf(pr, rL, pt * rV))));
+      const float vD = fmaf(up, Gp, fmaf(ub, Gb, ur * Gr));      // x (-1/dlambdaD)
+      const float vA = fmaf(SHp, alp, fmaf(SFp, bep, fmaf(SHb, alb, fmaf(SFb, beb,
                        fmaf(SHr, alr, SFr * ber)))));
-      float vV = Gp + Gb + Gr;                             // x kv
-#if !VFISV_FOLD_ID_IN_WEIGHTS
-      // the 1/Delta of every partial, applied to the six row values
-      vB *= iD; vG *= iD; vE *= iD; vD *= iD; vA *= iD; vV *= iD;
-#endif
-#pragma unroll
-      for (int k = 0; k < NF; ++k) {
-        acc[kRowB][S][k] = fmaf(Td[k], vB, acc[kRowB][S][k]);
-        acc[kRowG][S][k] = fmaf(Td[k], vG, acc[kRowG][S][k]);
-        acc[kRowE][S][k] = fmaf(Td[k], vE, acc[kRowE][S][k]);
-        acc[kRowD][S][k] = fmaf(Td[k], vD, acc[kRowD][S][k]);
-        acc[kRowA][S][k] = fmaf(Td[k], vA, acc[kRowA][S][k]);
-        acc[kRowV][S][k] = fmaf(Td[k], vV, acc[kRowV][S][k]);
-      }
+      const float vV = Gp + Gb + Gr;                             // x kv
+      out.rows(S, vB, vG, vE, vD, vA, vV);
     };
     // y_S = s N_S / Delta => Delta dy_S/dX = s dN_S/dX - y_S dDelta/dX
     stokes(0, fmaf(-yI, dDe, fmaf(3.0f, eI2, rr)), -yI * dDq, -yI * dDv,
@@ -295,12 +264,58 @@ __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, fl
       const float ny2 = -eta0 * yn * yn;
       const float nU = ny2 * bep;  // d/du_p
       const float nv[kNmRows] = {yn, ny2 * Hp, up * nU, ny2 * alp, nU};
+      out.nonmagnetic(nv);
+    }
+  }
+}
+
+// One wavelength point: synthesis (and, if DERIV, the Jacobian rows),
+// accumulated into acc[row][stokes][k] += T_k * value.
+template <int NF, bool DERIV, bool NM = false>
+__device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, float x,
+                                            const float (&T)[NF],
+                                            float (&acc)[DERIV ? kRows : 1][4][NF],
+                                            float (*accn)[NF] = nullptr) {
+  struct Sum {
+    const float (&T)[NF];
+    float (&acc)[DERIV ? kRows : 1][4][NF];
+    float (*accn)[NF];
+    // Weights of the derivative rows: the 1/Delta of every partial folded
+    // into the filter weight (6 products a point instead of 24).
+    float Td[NF];
+    __device__ __forceinline__ void unit(float yI, float yQ, float yU, float yV) {
+#pragma unroll
+      for (int k = 0; k < NF; ++k) {
+        acc[0][0][k] = fmaf(T[k], yI, acc[0][0][k]);
+        acc[0][1][k] = fmaf(T[k], yQ, acc[0][1][k]);
+        acc[0][2][k] = fmaf(T[k], yU, acc[0][2][k]);
+        acc[0][3][k] = fmaf(T[k], yV, acc[0][3][k]);
+      }
+    }
+    __device__ __forceinline__ void scale(float iD) {
+#pragma unroll
+      for (int k = 0; k < NF; ++k) Td[k] = T[k] * iD;
+    }
+    __device__ __forceinline__ void rows(int S, float vB, float vG, float vE, float vD, float vA,
+                                         float vV) {
+#pragma unroll
+      for (int k = 0; k < NF; ++k) {
+        acc[kRowB][S][k] = fmaf(Td[k], vB, acc[kRowB][S][k]);
+        acc[kRowG][S][k] = fmaf(Td[k], vG, acc[kRowG][S][k]);
+        acc[kRowE][S][k] = fmaf(Td[k], vE, acc[kRowE][S][k]);
+        acc[kRowD][S][k] = fmaf(Td[k], vD, acc[kRowD][S][k]);
+        acc[kRowA][S][k] = fmaf(Td[k], vA, acc[kRowA][S][k]);
+        acc[kRowV][S][k] = fmaf(Td[k], vV, acc[kRowV][S][k]);
+      }
+    }
+    __device__ __forceinline__ void nonmagnetic(const float (&nv)[kNmRows]) {
 #pragma unroll
       for (int k = 0; k < NF; ++k)
 #pragma unroll
         for (int r = 0; r < kNmRows; ++r) accn[r][k] = fmaf(T[k], nv[r], accn[r][k]);
     }
-  }
+  } sum{T, acc, accn, {}};
+  lambda_point<DERIV, NM>(W, P, x, sum);
 }
 
 }  // namespace vfisv
