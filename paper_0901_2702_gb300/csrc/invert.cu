@@ -1028,21 +1028,29 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
   }
   const bool plain = !restarts && !fast_solve;
   if (*block == 0) {
-    // no shape set: by the size of the map.  Up to twice the pixels that the
-    // kernel with several lanes a pixel holds at once (19,456 on 152 SMs) that
-    // kernel is the faster one -- 300 pixels 1.15 ms against 4.05 (128 x 1)
-    // and 5.35 (warp-specialised), 4,096 1.72 / 4.05 / 5.36, 12,288 3.46 /
-    // 4.07 / 5.33, 20,000 5.14 / 6.21 / 5.37 -- above it the warp-specialised
-    // one: 40,000 8.96 / 8.25 / 6.12, 1,048,576 204 / 138 / 101.
+    // no shape set: by the pixels an SM gets.  Several lanes a pixel up to
+    // 100 (15,200 pixels on 152 SMs), 128 x 1 while one CTA an SM holds the
+    // map, the warp-specialised kernel above.  Measured (ms; lanes / 128 x 1 /
+    // warp-specialised): 300 pixels 1.15 / 4.04 / 5.36, 4,096 1.64 / 4.06 /
+    // 5.37, 12,288 3.27 / 4.07 / 5.35, 19,000 5.38 / 4.08 / 5.37, 20,000 5.14
+    // / 6.21 / 5.37, 40,000 8.96 / 8.25 / 6.12, 1,048,576 204 / 138 / 101.
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    nsm = sm_budget(nsm);
     *block = kInvThreadsDefault;
+    *tpp = 1;
     if (plain) {
-      if (invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
+      // (a long filter table leaves room for few one-warp CTAs: those maps
+      // must then fit twice over)
+      if (npix <= 100 * (int64_t)nsm &&
+          invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
           npix <= 2 * *nslots)
         *block = kInvLanesBlock;
-      else if (invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
+      else if (npix > (int64_t)kInvThreadsDefault * nsm &&
+               invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
         *block = kInvWsBlock;
-      else
-        cudaGetLastError();
+      cudaGetLastError();
     }
   }
   if (*block == kInvLanesBlock || *block == kInvWsBlock) {

@@ -3,10 +3,11 @@
 // damped solve and chi2, filling factor held, no restarts).  T consecutive
 // lanes share a pixel, a CTA is one warp, and a call's time is the latency of
 // its longest chain of iterations; the lanes shorten every part of it:
-//   pass      lane q evaluates grid point step * T + q and puts its 28 values
-//             and 1/Delta into shared memory; then each lane adds the step's
-//             points, in grid order, to its own share of the 168 filtered
-//             sums (one Stokes parameter, 24 / T filters, 7 rows);
+//   pass      a step takes 2 T grid points: lane q evaluates points 2 q and
+//             2 q + 1 (packed) and puts their 28 values and 1/Delta into
+//             shared memory; then each lane adds the step's points, in grid
+//             order, to its own share of the 168 filtered sums (one Stokes
+//             parameter, 24 / T filters, 7 rows);
 //   chi2      a lane forms the FP64 products of its observables, every lane
 //             adds the 24 of them in order;
 //   normal    the lanes put the Jacobian rows of their observables into
@@ -26,6 +27,7 @@
 
 #include "common.cuh"
 #include "lm_device.cuh"
+#include "me_pair.cuh"
 #include "solve.cuh"
 
 namespace vfisv {
@@ -44,7 +46,7 @@ template <int T>
 struct LnSmem {
   static constexpr int P = 32 / T;  // pixels of a warp
   static constexpr int kPixRec = kLnObs * kLnRec + kLnRec;  // padded: no bank conflicts
-  static constexpr int kBuf = (kLnVals * 32 > P * kPixRec) ? kLnVals * 32 : P * kPixRec;
+  static constexpr int kBuf = (kLnVals * 64 > P * kPixRec) ? kLnVals * 64 : P * kPixRec;
   float buf[kBuf];              // point values, chi2 terms, observables' records (in turn)
   float scr[P][kNPk + kNP];     // normal equations of the best model
   float m[P][10], mt[P][10];    // best and trial model
@@ -53,35 +55,38 @@ struct LnSmem {
   uint64_t pad;
 };
 
-// Position of value v of point j of pixel p in the buffer: row v of 32
-// floats, its 16-byte pieces permuted so that lanes reading the same piece of
-// the rows of different Stokes parameters (v mod 4) meet different banks.
+// Position of value v of the step's point j (of 2 T) of pixel p in the
+// buffer: row v of 64 floats, its 16-byte pieces permuted so that lanes
+// reading the same piece of the rows of different Stokes parameters (v mod 4)
+// meet different banks.
 template <int T>
 __device__ __forceinline__ int ln_at(int v, int p, int j) {
-  const int c = (p * T + j) >> 2;
-  return v * 32 + (((c ^ (T == 4 ? 2 * (v & 3) : (v & 3))) << 2) | (j & 3));
+  const int c = (p * 2 * T + j) >> 2;
+  return v * 64 + (((c ^ (v & 3)) << 2) | (j & 3));
 }
 
-// Puts the values of lambda_point() into the buffer.
+// Puts the values of lambda_pair() (points j, j + 1) into the buffer.
 template <int T>
 struct LnPut {
   float* buf;
   int p, j;
-  __device__ __forceinline__ void unit(float yI, float yQ, float yU, float yV) {
-    buf[ln_at<T>(0, p, j)] = yI;
-    buf[ln_at<T>(1, p, j)] = yQ;
-    buf[ln_at<T>(2, p, j)] = yU;
-    buf[ln_at<T>(3, p, j)] = yV;
+  __device__ __forceinline__ void put(int v, f2 x) {
+    *reinterpret_cast<unsigned long long*>(buf + ln_at<T>(v, p, j)) = x.v;
   }
-  __device__ __forceinline__ void scale(float iD) { buf[ln_at<T>(4 * kRows, p, j)] = iD; }
-  __device__ __forceinline__ void rows(int S, float vB, float vG, float vE, float vD, float vA,
-                                       float vV) {
-    buf[ln_at<T>(4 * kRowB + S, p, j)] = vB;
-    buf[ln_at<T>(4 * kRowG + S, p, j)] = vG;
-    buf[ln_at<T>(4 * kRowE + S, p, j)] = vE;
-    buf[ln_at<T>(4 * kRowD + S, p, j)] = vD;
-    buf[ln_at<T>(4 * kRowA + S, p, j)] = vA;
-    buf[ln_at<T>(4 * kRowV + S, p, j)] = vV;
+  __device__ __forceinline__ void unit(f2 yI, f2 yQ, f2 yU, f2 yV) {
+    put(0, yI);
+    put(1, yQ);
+    put(2, yU);
+    put(3, yV);
+  }
+  __device__ __forceinline__ void scale(f2 iD) { put(4 * kRows, iD); }
+  __device__ __forceinline__ void rows(int S, f2 vB, f2 vG, f2 vE, f2 vD, f2 vA, f2 vV) {
+    put(4 * kRowB + S, vB);
+    put(4 * kRowG + S, vG);
+    put(4 * kRowE + S, vE);
+    put(4 * kRowD + S, vD);
+    put(4 * kRowA + S, vA);
+    put(4 * kRowV + S, vV);
   }
 };
 
@@ -95,15 +100,16 @@ __device__ __forceinline__ void ln_pass(const PixK& P, const float* __restrict__
   for (int r = 0; r < kRows; ++r)
 #pragma unroll
     for (int i = 0; i < KPL; ++i) acc[r][i] = 0.0f;
-  LnPut<T> put{buf, p, q};
+  LnPut<T> put{buf, p, 2 * q};
 #pragma unroll 1
-  for (int base = 0; base < nrows; base += T) {
+  for (int base = 0; base < nrows; base += 2 * T) {
     // past the last point: its values again, which nothing adds
-    const int i = min(base + q, nrows - 1);
-    lambda_point<true, false>(c_Wln, P, tab[(size_t)i * S + kLnNF], put);
+    const int i0 = min(base + 2 * q, nrows - 1), i1 = min(base + 2 * q + 1, nrows - 1);
+    lambda_pair<true>(c_Wln, P, f2_pack(tab[(size_t)i0 * S + kLnNF], tab[(size_t)i1 * S + kLnNF]),
+                      put);
     __syncwarp();
-#pragma unroll
-    for (int h = 0; h < T; h += 4) {
+#pragma unroll 1
+    for (int h = 0; h < 2 * T; h += 4) {
       float v[kRows][4], d[4];
 #pragma unroll
       for (int r = 0; r < kRows; ++r)

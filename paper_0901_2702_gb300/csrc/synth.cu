@@ -1,7 +1,7 @@
 // Milne-Eddington synthesis through the instrument filters (Secs. 3.1-3.2):
 // one pixel per thread, the filter/wavelength table in shared memory.
 #include "common.cuh"
-#include "f32x2.cuh"
+#include "me_pair.cuh"
 
 namespace vfisv {
 
@@ -170,71 +170,6 @@ cudaError_t launch_pack_table(const float* filters, int nf, const float* wl, int
   return cudaGetLastError();
 }
 
-// H(a,u) + i F(a,u) at two frequencies: faddeeva() with every operation on a
-// pair (the imaginary part of the Horner sum is carried negated, which is
-// exact, because the packed instructions take no negated operand).
-__device__ __forceinline__ void faddeeva_pair(const Weideman& W, f2 u, float a, f2& H, f2& F) {
-  const float L = W.L, lp = L + a;
-  const f2 lp2 = f2_dup(lp);
-  const f2 nu = f2_neg(u);
-  const f2 uu = f2_mul(u, nu);  // -u^2
-  const f2 dd = f2_fma(lp2, lp2, f2_mul(u, u));
-  const f2 rd = f2_pack(rcp_fast(f2_lo(dd)), rcp_fast(f2_hi(dd)));
-  const f2 zr = f2_mul(f2_fma(f2_dup(L - a), lp2, uu), rd);
-  const f2 nzi = f2_mul(f2_mul(f2_dup(2.0f * L), nu), rd);
-  const f2 zi = f2_neg(nzi);
-  // the first step (imaginary part zero) written out
-  f2 pr = f2_fma(f2_dup(W.a[kWeidN]), zr, f2_dup(W.a[kWeidN - 1]));
-  f2 npi = f2_mul(f2_dup(W.a[kWeidN]), nzi);
-#pragma unroll
-  for (int n = kWeidN - 2; n >= 1; --n) {
-    const f2 t = f2_fma(pr, zr, f2_fma(npi, zi, f2_dup(W.a[n])));
-    npi = f2_fma(pr, nzi, f2_mul(npi, zr));
-    pr = t;
-  }
-  const f2 qr = f2_mul(lp2, rd), qi = f2_mul(u, rd);  // 1/(L - iz)
-  const f2 q2r = f2_fma(qr, qr, f2_mul(f2_neg(qi), qi));
-  const f2 q2i = f2_mul(f2_mul(f2_dup(2.0f), qr), qi);
-  const f2 two = f2_dup(2.0f), is = f2_dup(kInvSqrtPi);
-  H = f2_fma(two, f2_fma(pr, q2r, f2_mul(npi, q2i)), f2_mul(is, qr));
-  F = f2_fma(two, f2_fma(pr, q2i, f2_mul(f2_neg(npi), q2r)), f2_mul(is, qi));
-}
-
-// Unit-S1 Stokes values (I, Q0, U0, V in the psi = 0 frame) at two
-// wavelength offsets: the synthesis half of lambda_step() on pairs.
-__device__ __forceinline__ void stokes_pair(const Weideman& W, const PixK& P, f2 x, f2 (&y)[4]) {
-  const f2 half = f2_dup(-0.5f);
-  const f2 up = f2_fma(x, f2_dup(P.invD), f2_dup(-P.uv));
-  const f2 ub = f2_add(up, f2_dup(P.uB)), ur = f2_sub(up, f2_dup(P.uB));
-  f2 Hp, Fp, Hb, Fb, Hr, Fr;
-  faddeeva_pair(W, up, P.a, Hp, Fp);
-  faddeeva_pair(W, ub, P.a, Hb, Fb);
-  faddeeva_pair(W, ur, P.a, Hr, Fr);
-  const f2 Hsum = f2_add(Hb, Hr), Hdif = f2_sub(Hr, Hb);
-  const f2 Fsum = f2_add(Fb, Fr), Fdif = f2_sub(Fr, Fb);
-  const f2 hL = f2_fma(half, Hsum, Hp), fL = f2_fma(half, Fsum, Fp);
-  const f2 c1 = f2_dup(P.c1), c4 = f2_dup(P.c4);
-  const f2 eI = f2_fma(c1, Hp, f2_fma(f2_dup(P.c2), Hsum, f2_dup(1.0f)));
-  const f2 eL = f2_mul(c1, hL), eV = f2_mul(c4, Hdif);
-  const f2 rL = f2_mul(c1, fL), rV = f2_mul(c4, Fdif);
-  const f2 eI2 = f2_mul(eI, eI);
-  const f2 Pi = f2_fma(eL, rL, f2_mul(eV, rV));
-  const f2 rr = f2_fma(rL, rL, f2_mul(rV, rV));
-  const f2 g = f2_add(f2_sub(eI2, f2_fma(eL, eL, f2_mul(eV, eV))), rr);
-  const f2 nPi = f2_neg(Pi);
-  const f2 Dl = f2_fma(eI2, g, f2_mul(nPi, Pi));
-  const f2 iD = f2_pack(rcp_fast(f2_lo(Dl)), rcp_fast(f2_hi(Dl)));
-  const f2 niD = f2_neg(iD);
-  const f2 NI = f2_mul(eI, f2_add(eI2, rr));
-  const f2 NQ = f2_fma(eI2, eL, f2_mul(rL, Pi));
-  const f2 NU = f2_mul(eI, f2_fma(eL, rV, f2_mul(f2_neg(eV), rL)));
-  const f2 NV = f2_fma(eI2, eV, f2_mul(rV, Pi));
-  y[0] = f2_mul(NI, iD);
-  y[1] = f2_mul(NQ, niD);
-  y[2] = f2_mul(NU, niD);
-  y[3] = f2_mul(NV, niD);
-}
-
 // Filtered unit-S1 Stokes values of one model.  Two wavelength points per
 // round, packed: the scalar loop issued 327 instructions a point and stalled
 // on dispatch with the FMA pipe 73 % active (1,048,576 pixels, 63 points:
@@ -252,8 +187,17 @@ __device__ __forceinline__ void synth_pixel(const Weideman& W, const PixK& P,
     float T0[NF], T1[NF];
     const float x0 = load_row<NF>(tab + (size_t)i * S, T0);
     const float x1 = load_row<NF>(tab + (size_t)(both ? i + 1 : i) * S, T1);
-    f2 y[4];
-    stokes_pair(W, P, f2_pack(x0, x1), y);
+    struct Take {
+      f2 y[4];
+      __device__ __forceinline__ void unit(f2 yI, f2 yQ, f2 yU, f2 yV) {
+        y[0] = yI;
+        y[1] = yQ;
+        y[2] = yU;
+        y[3] = yV;
+      }
+    } out;
+    lambda_pair<false>(W, P, f2_pack(x0, x1), out);
+    const f2 (&y)[4] = out.y;
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
