@@ -47,7 +47,7 @@ constexpr int kWsWarps = 12;
 constexpr int kWsThreadsN = kWsWarps * 32;
 constexpr int kWsBatches = 8;                  // consumer warps
 constexpr int kWsSlotsN = kWsBatches * 32;     // pixel slots per CTA
-constexpr int kWsProdRegs = 232, kWsConsRegs = 136;
+constexpr int kWsProdRegs = 240, kWsConsRegs = 128;
 constexpr int kWsTmemCols = 512;
 constexpr int kWsGroup = 8;                    // columns per (filter, Stokes) group
 constexpr int kWsBatchCols = 256;              // batch 1 of a producer starts here
@@ -195,7 +195,7 @@ __device__ __forceinline__ bool ws_producer(const InvertArgs& A, int p, uint32_t
         for (int i = 0; i < nrows; ++i) {
           float T[NF];
           const float xw = load_row<NF>(tab + (size_t)i * S, T);
-          lambda_step<NF, true>(c_Wws, P, xw, T, acc);
+          lambda_step<NF, true, false, true>(c_Wws, P, xw, T, acc);
         }
       }
       // every lane of the warp stores (the tensor-memory stores are

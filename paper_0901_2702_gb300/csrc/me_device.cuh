@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "f32x2.cuh"
+
 namespace vfisv {
 
 // Number of terms of the Weideman (1994) rational series for w(z).  With 16
@@ -67,6 +69,38 @@ __device__ __forceinline__ void faddeeva(const Weideman& W, float u, float a,
   const float q2r = fmaf(qr, qr, -qi * qi), q2i = 2.0f * qr * qi;
   H = fmaf(2.0f, fmaf(pr, q2r, -pi * q2i), kInvSqrtPi * qr);
   F = fmaf(2.0f, fmaf(pr, q2i, pi * q2r), kInvSqrtPi * qi);
+}
+
+__device__ __forceinline__ f2 f2_rcp_fast(f2 a) {
+  return f2_pack(rcp_fast(f2_lo(a)), rcp_fast(f2_hi(a)));
+}
+
+// H(a,u) + i F(a,u) at two frequencies (faddeeva(); the imaginary part of the
+// Horner sum is carried negated).
+__device__ __forceinline__ void faddeeva_pair(const Weideman& W, f2 u, float a, f2& H, f2& F) {
+  const float L = W.L, lp = L + a;
+  const f2 lp2 = f2_dup(lp);
+  const f2 nu = f2_neg(u);
+  const f2 uu = f2_mul(u, nu);  // -u^2
+  const f2 rd = f2_rcp_fast(f2_fma(lp2, lp2, f2_mul(u, u)));
+  const f2 zr = f2_mul(f2_fma(f2_dup(L - a), lp2, uu), rd);
+  const f2 nzi = f2_mul(f2_mul(f2_dup(2.0f * L), nu), rd);
+  const f2 zi = f2_neg(nzi);
+  // the first step (imaginary part zero) written out
+  f2 pr = f2_fma(f2_dup(W.a[kWeidN]), zr, f2_dup(W.a[kWeidN - 1]));
+  f2 npi = f2_mul(f2_dup(W.a[kWeidN]), nzi);
+#pragma unroll
+  for (int n = kWeidN - 2; n >= 1; --n) {
+    const f2 t = f2_fma(pr, zr, f2_fma(npi, zi, f2_dup(W.a[n])));
+    npi = f2_fma(pr, nzi, f2_mul(npi, zr));
+    pr = t;
+  }
+  const f2 qr = f2_mul(lp2, rd), qi = f2_mul(u, rd);  // 1/(L - iz)
+  const f2 q2r = f2_fma(qr, qr, f2_mul(f2_neg(qi), qi));
+  const f2 q2i = f2_mul(f2_mul(f2_dup(2.0f), qr), qi);
+  const f2 two = f2_dup(2.0f), is = f2_dup(kInvSqrtPi);
+  H = f2_fma(two, f2_fma(pr, q2r, f2_mul(npi, q2i)), f2_mul(is, qr));
+  F = f2_fma(two, f2_fma(pr, q2i, f2_mul(f2_neg(npi), q2r)), f2_mul(is, qi));
 }
 
 // Model bounds, applied after every step of the inversion and to initial
@@ -167,14 +201,24 @@ constexpr int kNmRows = 5;
 // the 1/Delta that every derivative row still lacks, then rows(S, vB, vG, vE,
 // vD, vA, vV) for each Stokes parameter S, and with NM the non-magnetic rows
 // nonmagnetic(v).
-template <bool DERIV, bool NM, class Out>
+// With BR the two sigma components run packed.
+template <bool DERIV, bool NM, bool BR = false, class Out>
 __device__ __forceinline__ void lambda_point(const Weideman& W, const PixK& P, float x, Out& out) {
   const float up = fmaf(x, P.invD, -P.uv);
   const float ub = up + P.uB, ur = up - P.uB;
   float Hp, Fp, Hb, Fb, Hr, Fr;
   faddeeva(W, up, P.a, Hp, Fp);
-  faddeeva(W, ub, P.a, Hb, Fb);
-  faddeeva(W, ur, P.a, Hr, Fr);
+  if constexpr (BR) {
+    f2 H, F;
+    faddeeva_pair(W, f2_pack(ub, ur), P.a, H, F);
+    Hb = f2_lo(H);
+    Hr = f2_hi(H);
+    Fb = f2_lo(F);
+    Fr = f2_hi(F);
+  } else {
+    faddeeva(W, ub, P.a, Hb, Fb);
+    faddeeva(W, ur, P.a, Hr, Fr);
+  }
   const float Hsum = Hb + Hr, Hdif = Hr - Hb;
   const float Fsum = Fb + Fr, Fdif = Fr - Fb;
   // absorption-matrix elements (psi = 0 frame)
@@ -271,7 +315,7 @@ __device__ __forceinline__ void lambda_point(const Weideman& W, const PixK& P, f
 
 // One wavelength point: synthesis (and, if DERIV, the Jacobian rows),
 // accumulated into acc[row][stokes][k] += T_k * value.
-template <int NF, bool DERIV, bool NM = false>
+template <int NF, bool DERIV, bool NM = false, bool BR = false>
 __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, float x,
                                             const float (&T)[NF],
                                             float (&acc)[DERIV ? kRows : 1][4][NF],
@@ -315,7 +359,7 @@ __device__ __forceinline__ void lambda_step(const Weideman& W, const PixK& P, fl
         for (int r = 0; r < kNmRows; ++r) accn[r][k] = fmaf(T[k], nv[r], accn[r][k]);
     }
   } sum{T, acc, accn, {}};
-  lambda_point<DERIV, NM>(W, P, x, sum);
+  lambda_point<DERIV, NM, BR>(W, P, x, sum);
 }
 
 }  // namespace vfisv

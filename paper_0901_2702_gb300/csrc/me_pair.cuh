@@ -5,42 +5,9 @@
 // operand), so a point's values are the same bits either way.
 #pragma once
 
-#include "f32x2.cuh"
 #include "me_device.cuh"
 
 namespace vfisv {
-
-__device__ __forceinline__ f2 f2_rcp_fast(f2 a) {
-  return f2_pack(rcp_fast(f2_lo(a)), rcp_fast(f2_hi(a)));
-}
-
-// H(a,u) + i F(a,u) at two frequencies (faddeeva(); the imaginary part of the
-// Horner sum is carried negated).
-__device__ __forceinline__ void faddeeva_pair(const Weideman& W, f2 u, float a, f2& H, f2& F) {
-  const float L = W.L, lp = L + a;
-  const f2 lp2 = f2_dup(lp);
-  const f2 nu = f2_neg(u);
-  const f2 uu = f2_mul(u, nu);  // -u^2
-  const f2 rd = f2_rcp_fast(f2_fma(lp2, lp2, f2_mul(u, u)));
-  const f2 zr = f2_mul(f2_fma(f2_dup(L - a), lp2, uu), rd);
-  const f2 nzi = f2_mul(f2_mul(f2_dup(2.0f * L), nu), rd);
-  const f2 zi = f2_neg(nzi);
-  // the first step (imaginary part zero) written out
-  f2 pr = f2_fma(f2_dup(W.a[kWeidN]), zr, f2_dup(W.a[kWeidN - 1]));
-  f2 npi = f2_mul(f2_dup(W.a[kWeidN]), nzi);
-#pragma unroll
-  for (int n = kWeidN - 2; n >= 1; --n) {
-    const f2 t = f2_fma(pr, zr, f2_fma(npi, zi, f2_dup(W.a[n])));
-    npi = f2_fma(pr, nzi, f2_mul(npi, zr));
-    pr = t;
-  }
-  const f2 qr = f2_mul(lp2, rd), qi = f2_mul(u, rd);  // 1/(L - iz)
-  const f2 q2r = f2_fma(qr, qr, f2_mul(f2_neg(qi), qi));
-  const f2 q2i = f2_mul(f2_mul(f2_dup(2.0f), qr), qi);
-  const f2 two = f2_dup(2.0f), is = f2_dup(kInvSqrtPi);
-  H = f2_fma(two, f2_fma(pr, q2r, f2_mul(npi, q2i)), f2_mul(is, qr));
-  F = f2_fma(two, f2_fma(pr, q2i, f2_mul(f2_neg(npi), q2r)), f2_mul(is, qi));
-}
 
 // lambda_point() at the offsets x: `out` gets the same calls with pairs.
 template <bool DERIV, class Out>
