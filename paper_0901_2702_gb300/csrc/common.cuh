@@ -241,8 +241,8 @@ cudaError_t launch_restart_perturb(const float* in, int64_t n, int64_t pix0, int
 // current device (once per device).
 cudaError_t invert_set_constants(const Weideman& W);
 // The warp-specialised LM kernel (invert_ws.cu): CTAs of kInvWsBlock threads
-// (one producer warpgroup, two consumer warpgroups), 256 pixel slots each,
-// one per SM; the default configuration only (6 filters, FP64 solve, no
+// (a producer, an accumulator and a solver warpgroup), up to 384 pixel slots
+// each, one per SM; the default configuration only (6 filters, FP64 solve, no
 // restarts, filling factor held).
 constexpr int kInvWsBlock = 384;
 cudaError_t invert_ws_set_constants(const Weideman& W);

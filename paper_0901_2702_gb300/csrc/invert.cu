@@ -1029,11 +1029,11 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
   const bool plain = !restarts && !fast_solve;
   if (*block == 0) {
     // no shape set: by the pixels an SM gets.  Several lanes a pixel up to
-    // 100 (15,200 pixels on 152 SMs), 128 x 1 while one CTA an SM holds the
-    // map, the warp-specialised kernel above.  Measured (ms; lanes / 128 x 1 /
-    // warp-specialised): 300 pixels 1.15 / 4.04 / 5.36, 4,096 1.64 / 4.06 /
-    // 5.37, 12,288 3.27 / 4.07 / 5.35, 19,000 5.38 / 4.08 / 5.37, 20,000 5.14
-    // / 6.21 / 5.37, 40,000 8.96 / 8.25 / 6.12, 1,048,576 204 / 138 / 101.
+    // 100 (15,200 pixels on 152 SMs), the warp-specialised kernel above.
+    // Measured (ms; lanes / 128 x 1 / warp-specialised): 300 pixels 1.16 /
+    // 3.82 / 3.73, 4,096 1.64 / 4.06 / -, 12,288 3.26 / 3.85 / 3.77, 17,000
+    // - / 3.86 / 3.77, 19,000 5.38 / 3.86 / 3.77, 40,000 8.96 / 8.06 / 6.64,
+    // 1,048,576 204 / 138 / 85.
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1047,8 +1047,7 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
           invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
           npix <= 2 * *nslots)
         *block = kInvLanesBlock;
-      else if (npix > (int64_t)kInvThreadsDefault * nsm &&
-               invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
+      else if (invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
         *block = kInvWsBlock;
       cudaGetLastError();
     }

@@ -4,32 +4,41 @@
 // iteration, same arithmetic and same results as invert_kernel; only the
 // division of the work between warps differs.
 //
-// One CTA per SM, 384 threads in three warpgroups.  Warpgroup 0 (one warp
-// per SM sub-partition) only runs the fused FP32 synthesis + Jacobian +
-// filter pass over the wavelength grid (Secs. 3, 4.4).  Warpgroups 1 and 2
-// own the pixel slots, one per thread, and run everything else: the FP64
-// chi2 and the acceptance test (Eq. 1, Fig. 6), the compensated J^T W J
-// build (Eqs. 3-4), the FP64 damped solve (Eqs. 4-5), retirement and the
-// work queue.  Producer warp p serves consumer warps 4 + p and 8 + p (its
-// batches 0 and 1, 32 slots each) in turn: while it synthesises one batch's
-// trial models, the other batch's consumer warp works through its last
-// pass, so the FP32 pipe, the FP64 pipe and the latency of the solve
-// overlap in every sub-partition.
+// One CTA per SM, 384 threads in three warpgroups, one warp of each in every
+// SM sub-partition, working as a pipeline over up to three batches of 32
+// pixel slots:
+//   producer      the fused FP32 synthesis + Jacobian + filter pass over the
+//                 wavelength grid (Secs. 3, 4.4) at a batch's trial models;
+//   accumulator   the FP64 chi2 and the acceptance test (Eq. 1, Fig. 6), the
+//                 compensated J^T W J build (Eqs. 3-4), retirement and the
+//                 work queue;
+//   solver        the FP64 damped solve (Eqs. 4-5): the next trial models.
+// A batch is with one of the three at a time, so the FP32 pipe, the FP64 pipe
+// and the latencies of the sums and of the solve overlap in every
+// sub-partition.  With two warps that each took a batch through accumulation
+// and solve, a batch's own chain set the pace: 68 k cycles of pass and 123 to
+// 142 k of the rest, the producer idle a third of the time (1,048,576 pixels
+// 93.5 ms, FMA pipe 61 %).  Here the three stages take about 80 k cycles a
+// batch each, all busy, against one another (85.3 ms, FMA pipe 68 %): what
+// bounds them is the FP32 issue of producer and accumulator together and the
+// instruction cache, which three different streams share.  The solver's rolled
+// loops are for that: unrolled, its tens of KB of code stalled the other
+// warps' fetches (0.47 stalls an issue for lack of an instruction, 97 ms), and
+// half unrolled it was faster by itself and the kernel slower (90 ms).
 //
-// The 168 filtered rows of a pass go from producer to consumer through
-// tensor memory: producer lane l of warp p writes TMEM lane 32p + l, in the
-// batch's column range; consumer warps 4 + p and 8 + p sit in the same
-// sub-partition (warp id mod 4) and read the same lanes.  Within a batch's
-// range, the seven rows of Stokes s of filter k fill the 8-column group
-// k * 4 + s (row r at column r), and the unit-S1 Stokes values of all
-// observables follow contiguously for the chi2.  The slots' LM state
-// (models, normal equations, damping, best chi2, iteration, flags) lives in
-// shared memory.  Hand-offs are mbarriers with bounded waits: full[b] (rows
-// of batch b written), empty[b] (rows read and the next trial models of
-// batch b written).  Registers: the
-// producers raise their limit to 232 (the pass's accumulators without
-// spills), the consumers drop to 136 (setmaxnreg): three warps per
-// sub-partition against two for invert_kernel.
+// The 168 filtered rows of a pass go from producer to accumulator through
+// tensor memory: the three warps of a sub-partition (warp id mod 4) reach the
+// same 32 lanes, lane l of a warp holding slot l of its batch.  Passes
+// alternate between two column ranges.  Within a range, the seven rows of
+// Stokes s of filter k fill the 8-column group k * 4 + s (row r at column r),
+// and the unit-S1 Stokes values of all observables follow contiguously for
+// the chi2.  The slots' LM state (models, normal equations, damping, best
+// chi2, iteration, flags) lives in shared memory.  Hand-offs are mbarriers
+// with bounded waits, per sub-partition: full[2] (rows of a range written),
+// free[2] (rows read), ready[3] (a batch's trial models written), done[3] (a
+// batch's normal equations and new pixels written).  Registers: the producers
+// raise their limit to hold the pass's accumulators without spills, the
+// others drop (setmaxnreg).
 #include <math.h>
 
 #include "common.cuh"
@@ -45,40 +54,58 @@ namespace {
 
 constexpr int kWsWarps = 12;
 constexpr int kWsThreadsN = kWsWarps * 32;
-constexpr int kWsBatches = 8;                  // consumer warps
-constexpr int kWsSlotsN = kWsBatches * 32;     // pixel slots per CTA
-constexpr int kWsProdRegs = 240, kWsConsRegs = 128;
+constexpr int kWsGroups = 4;                   // SM sub-partitions
+constexpr int kWsBatches = 3;                  // batches of a sub-partition
+// pixel slots of a CTA with NB batches a sub-partition (two where a long
+// filter table leaves no room for three)
+template <int NB>
+constexpr int kWsSlots = kWsGroups * NB * 32;
+// The solver's matrix is in shared memory, or (no room beside a long table) in
+// registers; registers of the three kinds of warps accordingly.  Measured with
+// the matrix in shared memory, 1,048,576 pixels: 240 / 168 / 88 85.3 ms,
+// 240 / 160 / 96 85.4, 240 / 168 / 96 85.6, 232 / 168 / 96 87.4, 248 / 168 / 80
+// 89.0, 240 / 136 / 128 96.7.
+template <int NB>
+constexpr bool kSmemSolve = NB == kWsBatches;
+constexpr int kProdRegs = 240;
+template <int NB>
+constexpr int kAccRegs = kSmemSolve<NB> ? 168 : 128;
+template <int NB>
+constexpr int kSolveRegs = kSmemSolve<NB> ? 88 : 128;
 constexpr int kWsTmemCols = 512;
 constexpr int kWsGroup = 8;                    // columns per (filter, Stokes) group
-constexpr int kWsBatchCols = 256;              // batch 1 of a producer starts here
+constexpr int kWsRangeCols = 256;              // the second column range starts here
+constexpr int kWsBars = 4 + 2 * kWsBatches;    // full[2], free[2], ready[3], done[3]
 constexpr int kFlagNear = 1, kFlagFresh = 2;
-static_assert(kWsWarps == 4 + kWsBatches, "one producer warp per sub-partition");
-static_assert(kWsBatches == 8, "each producer warp serves two consumer warps");
-// a batch's 7-row groups and its row-0 copy fit its column range, and both
-// batches fit the allocation (a power of two, at most 512 columns)
-static_assert(4 * 6 * kWsGroup + 4 * 6 <= kWsBatchCols, "batch columns");
-static_assert(kWsBatchCols + 4 * 6 * kWsGroup + 4 * 6 <= kWsTmemCols && kWsTmemCols <= 512,
+static_assert(kWsWarps == 3 * kWsGroups, "one warp of each kind per sub-partition");
+// a pass's 7-row groups and its row-0 copy fit its column range, and both
+// ranges fit the allocation (a power of two, at most 512 columns)
+static_assert(4 * 6 * kWsGroup + 4 * 6 <= kWsRangeCols, "range columns");
+static_assert(kWsRangeCols + 4 * 6 * kWsGroup + 4 * 6 <= kWsTmemCols && kWsTmemCols <= 512,
               "tensor-memory columns");
-static_assert(kWsProdRegs % 8 == 0 && kWsConsRegs % 8 == 0, "setmaxnreg counts");
-
 // Shared-memory layout: the filter table, then these arrays (byte offsets
 // from the start of shared memory), structure of arrays over the slots.
+template <int NB>
 struct WsSmem {
-  size_t mt, m, scr, pix, eps, chi2, it, flags, fin, cnt, tslot, bars, tbar, total;
+  static constexpr int SL = kWsSlots<NB>;
+  size_t mt, m, scr, pix, eps, chi2, it, flags, fin, seq, sol, cnt, tslot, bars, tbar, total;
   __host__ __device__ explicit WsSmem(int tabf) {
     size_t o = (size_t)tabf * 4;
-    mt = o;   o += (size_t)10 * kWsSlotsN * 4;          // trial models [10][slots]
-    m = o;    o += (size_t)10 * kWsSlotsN * 4;          // best models [10][slots]
-    scr = o;  o += (size_t)(kNPk + kNP) * kWsSlotsN * 4;  // normal equations [54][slots]
-    pix = o;  o += (size_t)kWsSlotsN * 8;               // pixel of each slot (-1: idle)
-    eps = o;  o += (size_t)kWsSlotsN * 8;               // damping
-    chi2 = o; o += (size_t)kWsSlotsN * 8;               // chi2 of the best model
-    it = o;   o += (size_t)kWsSlotsN * 4;               // iterations
-    flags = o; o += (size_t)kWsSlotsN * 4;              // kFlagNear | kFlagFresh
+    mt = o;   o += (size_t)10 * SL * 4;          // trial models [10][slots]
+    m = o;    o += (size_t)10 * SL * 4;          // best models [10][slots]
+    scr = o;  o += (size_t)(kNPk + kNP) * SL * 4;  // normal equations [54][slots]
+    pix = o;  o += (size_t)SL * 8;               // pixel of each slot (-1: idle)
+    eps = o;  o += (size_t)SL * 8;               // damping
+    chi2 = o; o += (size_t)SL * 8;               // chi2 of the best model
+    it = o;   o += (size_t)SL * 4;               // iterations
+    flags = o; o += (size_t)SL * 4;              // kFlagNear | kFlagFresh
     fin = o;  o += 16 * 4;                               // batch finished flags
+    seq = o;  o += 2 * kWsGroups * 4;                    // batch of the pass in each range
+    sol = o;  // the solvers' matrices
+    if (kSmemSolve<NB>) o += (size_t)kWsGroups * (kNPk + kNP) * 32 * 8;
     cnt = o;  o += 4 * 8;                                // work counters
     tslot = o; o += 16;                                  // tensor-memory base address
-    bars = o; o += 2 * kWsBatches * 8;                   // full[8], empty[8]
+    bars = o; o += (size_t)kWsGroups * kWsBars * 8;      // hand-off barriers
     tbar = o; o += 16;                                   // table copy
     total = o;
   }
@@ -156,30 +183,59 @@ __device__ __forceinline__ void tm_wait24(uint32_t (&a)[8], uint32_t (&b)[8], ui
                  "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7])::"memory");
 }
 
-template <int NF>
-__device__ __forceinline__ bool ws_producer(const InvertArgs& A, int p, uint32_t tlane,
+// The barriers of a sub-partition.
+struct WsBars {
+  uint32_t base;
+  __device__ __forceinline__ uint32_t full(int r) const { return base + 8 * r; }
+  __device__ __forceinline__ uint32_t free(int r) const { return base + 8 * (2 + r); }
+  __device__ __forceinline__ uint32_t ready(int b) const { return base + 8 * (4 + b); }
+  __device__ __forceinline__ uint32_t done(int b) const {
+    return base + 8 * (4 + kWsBatches + b);
+  }
+};
+
+// fin and seq: this sub-partition's batch finished flags and the batch of the
+// pass in each column range (-1: no more passes).
+template <int NF, int NB>
+__device__ __forceinline__ bool ws_producer(const InvertArgs& A, int g, int nb, uint32_t tlane,
                                             const float* __restrict__ tab, int nrows,
                                             const float* sMt, const long long* sPix,
-                                            const int* fin, uint32_t bar_full,
-                                            uint32_t bar_empty) {
+                                            const int* fin, int* seq, WsBars bar) {
   constexpr int S = ((NF + 1) + 3) & ~3;
-  constexpr int NOBS = 4 * NF;
+  constexpr int NOBS = 4 * NF, SL = kWsSlots<NB>;
   const int lane = threadIdx.x & 31;
-  uint32_t pe = 0u, done = 0u;  // bit x: parity of batch x's empty barrier; batch x finished
-  while (done != 3u) {
-#pragma unroll 1
-    for (int x = 0; x < 2; ++x) {
-      if ((done >> x) & 1u) continue;
-      const int b = p + 4 * x;
-      if (!ws_wait(bar_empty + 8 * b, (pe >> x) & 1u)) return false;
-      pe ^= 1u << x;
+  uint32_t pr = 0u, pf = 0u;  // parities of ready[] and free[]
+  uint32_t alive = (1u << nb) - 1u;
+  int rng = 0;
+  // the batch of the next pass, in turn; -1 when all are finished; -2: a wait gave up
+  auto next_batch = [&](int b) {
+    while (alive) {
+      b = (b + 1 >= nb) ? 0 : b + 1;
+      if (!((alive >> b) & 1u)) continue;
+      if (!ws_wait(bar.ready(b), (pr >> b) & 1u)) return -2;
+      pr ^= 1u << b;
       __syncwarp();
-      tc_after();
-      if (*(volatile const int*)(fin + b)) {
-        done |= 1u << x;
-        continue;
-      }
-      const int slot = b * 32 + lane;
+      if (!*(volatile const int*)(fin + b)) return b;
+      alive &= ~(1u << b);
+    }
+    return -1;
+  };
+  for (int b = -1;;) {
+    b = next_batch(b);
+    if (b == -2) return false;
+    // the range's rows have been read (its first use waits for nothing)
+    if (!ws_wait(bar.free(rng), ((pf >> rng) & 1u) ^ 1u)) return false;
+    pf ^= 1u << rng;
+    __syncwarp();
+    tc_after();
+    if (lane == 0) *(volatile int*)(seq + rng) = b;
+    if (b < 0) {
+      __syncwarp();
+      ws_arrive(bar.full(rng));
+      return true;
+    }
+    {
+      const int slot = (g * NB + b) * 32 + lane;
       float acc[kRows][4][NF];
 #pragma unroll
       for (int r = 0; r < kRows; ++r)
@@ -188,9 +244,9 @@ __device__ __forceinline__ bool ws_producer(const InvertArgs& A, int p, uint32_t
 #pragma unroll
           for (int k = 0; k < NF; ++k) acc[r][s][k] = 0.0f;
       if (sPix[slot] >= 0) {
-        const PixK P = make_pixk(A.lk, sMt[0 * kWsSlotsN + slot], sMt[1 * kWsSlotsN + slot],
-                                 sMt[3 * kWsSlotsN + slot], sMt[4 * kWsSlotsN + slot],
-                                 sMt[5 * kWsSlotsN + slot], sMt[6 * kWsSlotsN + slot]);
+        const PixK P = make_pixk(A.lk, sMt[0 * SL + slot], sMt[1 * SL + slot],
+                                 sMt[3 * SL + slot], sMt[4 * SL + slot],
+                                 sMt[5 * SL + slot], sMt[6 * SL + slot]);
 #pragma unroll 1
         for (int i = 0; i < nrows; ++i) {
           float T[NF];
@@ -201,7 +257,7 @@ __device__ __forceinline__ bool ws_producer(const InvertArgs& A, int p, uint32_t
       // every lane of the warp stores (the tensor-memory stores are
       // warp-wide); idle slots store zeros
       __syncwarp();
-      const uint32_t tb = tlane + (x ? (uint32_t)kWsBatchCols : 0u);
+      const uint32_t tb = tlane + (rng ? (uint32_t)kWsRangeCols : 0u);
 #pragma unroll
       for (int k = 0; k < NF; ++k)
 #pragma unroll
@@ -218,44 +274,35 @@ __device__ __forceinline__ bool ws_producer(const InvertArgs& A, int p, uint32_t
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       tc_before();
       __syncwarp();
-      ws_arrive(bar_full + 8 * b);
+      ws_arrive(bar.full(rng));
     }
+    rng ^= 1;
   }
-  return true;
 }
 
-template <int NF>
-__device__ __forceinline__ bool ws_consumer(const InvertArgs& A, int b, uint32_t tc,
-                                            const float* __restrict__ tab, int nrows,
-                                            float* sMt, float* sM, float* sScr, long long* sPix,
-                                            double* sEps, double* sChi, int* sIt, int* sFlags,
-                                            int* fin, unsigned long long* cnt, uint32_t bar_full,
-                                            uint32_t bar_empty) {
+template <int NF, int NB>
+__device__ __forceinline__ bool ws_accumulator(const InvertArgs& A, int g, int nb, uint32_t tlane,
+                                               const float* __restrict__ tab, int nrows,
+                                               float* sMt, float* sM, float* sScr,
+                                               long long* sPix, double* sEps, double* sChi,
+                                               int* sIt, int* sFlags, int* fin, const int* seq,
+                                               unsigned long long* cnt, WsBars bar) {
   constexpr int NOBS = 4 * NF;
   constexpr int NP = kNP, NPK = kNPk;
-  constexpr int64_t ns = kWsSlotsN;
+  constexpr int SL = kWsSlots<NB>;
+  constexpr int64_t ns = SL;
   static_assert(NF == 6, "the tensor-memory layout holds 6 filter positions");
   const int lane = threadIdx.x & 31;
-  const int slot = b * 32 + lane;
-  float* Mt = sMt + slot;
-  float* M = sM + slot;
-  float* scr = sScr + slot;
   const float* tau = tab + (size_t)A.nlam * table_stride(NF);
   const int dof = NOBS - A.nfree;
   const int64_t npix = A.npix_dev ? *A.npix_dev : A.npix;
-  // the slot's LM state stays in shared memory between passes (fewer live
-  // registers beside the FP64 solve)
-  long long pix = -1;
 
-  // the next pixel of the queue into this slot: its starting model as the
-  // trial model (bad inputs are answered on the spot); -1 when none is left
-  auto next_pixel = [&]() {
+  // the next pixel of the queue into a slot: its starting model as the trial
+  // model (bad inputs are answered on the spot); -1 when none is left
+  auto next_pixel = [&](int slot) -> long long {
     for (;;) {
       const unsigned long long q = atomicAdd(A.queue, 1ull);
-      if ((long long)q >= npix) {
-        pix = -1;
-        return;
-      }
+      if ((long long)q >= npix) return -1;
       const long long pq = A.pix_list ? A.pix_list[q] : (long long)q;
       const float* o = A.obs + pq * NOBS;
       const float* wv = weight_row(A, pq, NOBS);
@@ -297,29 +344,42 @@ __device__ __forceinline__ bool ws_consumer(const InvertArgs& A, int b, uint32_t
         continue;
       }
 #pragma unroll
-      for (int j = 0; j < 10; ++j) Mt[j * kWsSlotsN] = m[j];
-      pix = pq;
+      for (int j = 0; j < 10; ++j) sMt[j * SL + slot] = m[j];
       sIt[slot] = 0;
       sEps[slot] = A.eps0;
       sFlags[slot] = kFlagFresh;
-      return;
+      return pq;
     }
   };
 
-  next_pixel();
-  sPix[slot] = pix;
-  bool any = __any_sync(0xffffffffu, pix >= 0);
-  if (!any && lane == 0) fin[b] = 1;
-  __syncwarp();
-  ws_arrive(bar_empty + 8 * b);
-  if (!any) return true;
-  uint32_t pf = 0u;
-  for (;;) {
-    if (!ws_wait(bar_full + 8 * b, pf)) return false;
-    pf ^= 1u;
+  // hands a batch's slots (their pixels, trial models or normal equations) on
+  // to the solver; the batch is finished when none holds a pixel
+  auto hand_on = [&](int b, int slot, long long pix) {
+    sPix[slot] = pix;
+    const bool any = __any_sync(0xffffffffu, pix >= 0);
+    if (!any && lane == 0) fin[b] = 1;
     __syncwarp();
+    ws_arrive(bar.done(b));
+  };
+  for (int b = 0; b < nb; ++b) {
+    const int slot = (g * NB + b) * 32 + lane;
+    hand_on(b, slot, next_pixel(slot));
+  }
+  uint32_t pf = 0u;  // parities of full[]
+  for (int rng = 0;; rng ^= 1) {
+    if (!ws_wait(bar.full(rng), (pf >> rng) & 1u)) return false;
+    pf ^= 1u << rng;
+    __syncwarp();
+    const int b = *(volatile const int*)(seq + rng);
+    if (b < 0) return true;
     tc_after();
     __syncwarp();
+    const uint32_t tc = tlane + (rng ? (uint32_t)kWsRangeCols : 0u);
+    const int slot = (g * NB + b) * 32 + lane;
+    float* Mt = sMt + slot;
+    float* M = sM + slot;
+    float* scr = sScr + slot;
+    long long pix = sPix[slot];
     // unit-S1 Stokes of every observable (warp-wide loads)
     uint32_t y0[NOBS];
     {
@@ -344,9 +404,9 @@ __device__ __forceinline__ bool ws_consumer(const InvertArgs& A, int b, uint32_t
       double eps = sEps[slot];
       const double chi2b = sChi[slot];
       // ---- model, residual and chi-square (Eq. 1, FP64) ----
-      sincosf(2.0f * Mt[2 * kWsSlotsN] * kDeg, &s2p, &c2p);
-      mus1 = A.lk.mu * Mt[8 * kWsSlotsN];
-      s0 = Mt[7 * kWsSlotsN];
+      sincosf(2.0f * Mt[2 * SL] * kDeg, &s2p, &c2p);
+      mus1 = A.lk.mu * Mt[8 * SL];
+      s0 = Mt[7 * SL];
       float syn[NOBS];
 #pragma unroll
       for (int k = 0; k < NF; ++k) {
@@ -433,20 +493,24 @@ __device__ __forceinline__ bool ws_consumer(const InvertArgs& A, int b, uint32_t
           }
         }
       } fetch{tc, o, wv, {}, {}, {}};
-      const RowScale R = row_scale(A.lk, live ? Mt[3 * kWsSlotsN] : 1.0f,
-                                   live ? Mt[4 * kWsSlotsN] : 1.0f);
+      const RowScale R = row_scale(A.lk, live ? Mt[3 * SL] : 1.0f,
+                                   live ? Mt[4 * SL] : 1.0f);
       build_normal_equations<NF, NP, false, true>(
           fetch, tau, scr, ns, mus1, c2p, s2p, s0, 1.0f, A.lk.mu, R, keepA, accept);
     }
+    // the rows have been read: the range takes the next pass but one
+    tc_before();
+    __syncwarp();
+    ws_arrive(bar.free(rng));
     if (live) {
       if (accept) {
 #pragma unroll
-        for (int j = 0; j < 10; ++j) M[j * kWsSlotsN] = Mt[j * kWsSlotsN];
+        for (int j = 0; j < 10; ++j) M[j * SL] = Mt[j * SL];
       }
       if (retire) {
         const bool nan = status == VFISV_PIX_NAN_STATE;
         const float* src = nan ? Mt : M;
-        for (int j = 0; j < 10; ++j) A.params_out[pix * 10 + j] = src[j * kWsSlotsN];
+        for (int j = 0; j < 10; ++j) A.params_out[pix * 10 + j] = src[j * SL];
         A.chi2_out[pix] = (float)(nan ? c2 : sChi[slot]);
         A.iters_out[pix] = sIt[slot];
         A.status_out[pix] = status;
@@ -474,36 +538,64 @@ __device__ __forceinline__ bool ws_consumer(const InvertArgs& A, int b, uint32_t
         }
         map_retired(A, pix);
         atomicAdd(&cnt[2], 1ull);
-        next_pixel();
-      } else {
-        // ---- next trial model: FP64 damped solve (Eqs. 3-5) ----
-        double d[NP];
-        damped_step_fp64_body<NP, true>(scr, ns, A.free_mask, sEps[slot], d);
-        float m[10];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) m[j] = (float)((double)M[j * kWsSlotsN] + d[j]);
-        m[9] = 1.0f;
-        apply_bounds(m);
-#pragma unroll
-        for (int j = 0; j < 10; ++j) Mt[j * kWsSlotsN] = m[j];
+        pix = next_pixel(slot);
       }
     }
-    sPix[slot] = pix;
-    any = __any_sync(0xffffffffu, pix >= 0);
-    if (!any && lane == 0) fin[b] = 1;
-    tc_before();
-    __syncwarp();
-    ws_arrive(bar_empty + 8 * b);
-    if (!any) return true;
+    hand_on(b, slot, pix);
   }
 }
 
-template <int NF>
-__global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A) {
+// The FP64 damped solve (Eqs. 3-5) of every batch handed on: the next trial
+// models of the slots whose pixel goes on (new pixels have theirs).
+template <int NB>
+__device__ __forceinline__ bool ws_solver(const InvertArgs& A, int g, int nb, float* sMt,
+                                          const float* sM, const float* sScr,
+                                          const long long* sPix, const double* sEps,
+                                          const int* sFlags, const int* fin, double* sSol, WsBars bar) {
+  constexpr int NP = kNP, SL = kWsSlots<NB>;
+  const int lane = threadIdx.x & 31;
+  uint32_t pd = 0u, alive = (1u << nb) - 1u;
+  for (int b = -1; alive;) {
+    b = (b + 1 >= nb) ? 0 : b + 1;
+    if (!((alive >> b) & 1u)) continue;
+    if (!ws_wait(bar.done(b), (pd >> b) & 1u)) return false;
+    pd ^= 1u << b;
+    __syncwarp();
+    const int slot = (g * NB + b) * 32 + lane;
+    if (*(volatile const int*)(fin + b)) {
+      alive &= ~(1u << b);
+    } else if (sPix[slot] >= 0 && !(sFlags[slot] & kFlagFresh)) {
+      if constexpr (kSmemSolve<NB>) {
+        damped_step_smem<NP>(sScr + slot, SL, A.free_mask, sEps[slot], sSol + lane, sM + slot,
+                             sMt + slot);
+      } else {
+        double d[NP];
+        damped_step_fp64_body<NP, true>(sScr + slot, SL, A.free_mask, sEps[slot], d);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) sMt[j * SL + slot] = (float)((double)sM[j * SL + slot] + d[j]);
+      }
+      float m[10];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) m[j] = sMt[j * SL + slot];
+      m[9] = 1.0f;
+      apply_bounds(m);
+#pragma unroll
+      for (int j = 0; j < 10; ++j) sMt[j * SL + slot] = m[j];
+    }
+    __syncwarp();
+    ws_arrive(bar.ready(b));
+  }
+  return true;
+}
+
+template <int NF, int NB>
+__global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A, int nb) {
+  static_assert(kProdRegs % 8 == 0 && kAccRegs<NB> % 8 == 0 && kSolveRegs<NB> % 8 == 0,
+                "setmaxnreg counts");
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int tabf = table_floats(NF, A.nlam);
-  const WsSmem L(tabf);
+  const WsSmem<NB> L(tabf);
   char* base = reinterpret_cast<char*>(smem);
   float* tab = smem;
   float* sMt = reinterpret_cast<float*>(base + L.mt);
@@ -517,13 +609,14 @@ __global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A)
   int* fin = reinterpret_cast<int*>(base + L.fin);
   unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + L.cnt);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(base + L.tslot);
-  const uint32_t bar_full = smem_u32(base + L.bars), bar_empty = bar_full + 8 * kWsBatches;
+  int* seq = reinterpret_cast<int*>(base + L.seq);
+  const uint32_t bars = smem_u32(base + L.bars);
   if (tid == 0) {
-    for (int i = 0; i < 2 * kWsBatches; ++i)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar_full + 8 * i), "r"(32)
+    for (int i = 0; i < kWsGroups * kWsBars; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bars + 8 * i), "r"(32)
                    : "memory");
   }
-  if (tid < kWsBatches) fin[tid] = 0;
+  if (tid < kWsGroups * NB) fin[tid] = 0;
   if (tid < 4) cnt[tid] = 0;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -543,17 +636,23 @@ __global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A)
   const int nrows = table_rows(tab, NF, A.nlam);
   bool good = true;
   if (ok) {
-    if (warp < 4) {
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWsProdRegs));
-      good = ws_producer<NF>(A, warp, tmem + ((uint32_t)(32 * warp) << 16), tab, nrows, sMt,
-                             sPix, fin, bar_full, bar_empty);
+    const int g = warp & 3;  // sub-partition
+    const WsBars bar{bars + (uint32_t)(8 * kWsBars * g)};
+    const uint32_t tlane = tmem + ((uint32_t)(32 * g) << 16);
+    int* gfin = fin + g * NB;
+    int* gseq = seq + 2 * g;
+    double* sSol = reinterpret_cast<double*>(base + L.sol) + (size_t)g * (kNPk + kNP) * 32;
+    const int role = warp >> 2;
+    if (role == 0) {
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kProdRegs));
+      good = ws_producer<NF, NB>(A, g, nb, tlane, tab, nrows, sMt, sPix, gfin, gseq, bar);
+    } else if (role == 1) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kAccRegs<NB>));
+      good = ws_accumulator<NF, NB>(A, g, nb, tlane, tab, nrows, sMt, sM, sScr, sPix, sEps, sChi, sIt,
+                                sFlags, gfin, gseq, cnt, bar);
     } else {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWsConsRegs));
-      const int b = warp - 4;  // batch: producer b % 4, its batch b / 4
-      const uint32_t tc = tmem + ((uint32_t)(32 * (b & 3)) << 16) +
-                          ((b >> 2) ? (uint32_t)kWsBatchCols : 0u);
-      good = ws_consumer<NF>(A, b, tc, tab, nrows, sMt, sM, sScr, sPix, sEps, sChi, sIt, sFlags,
-                             fin, cnt, bar_full, bar_empty);
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kSolveRegs<NB>));
+      good = ws_solver<NB>(A, g, nb, sMt, sM, sScr, sPix, sEps, sFlags, gfin, sSol, bar);
     }
   }
   if (!good) atomicExch(A.err, kDevErrWsWait);
@@ -574,41 +673,63 @@ cudaError_t invert_ws_set_constants(const Weideman& W) {
   return cudaMemcpyToSymbol(c_Wws, &W, sizeof(W));
 }
 
-size_t invert_ws_smem_bytes(int nlam) { return WsSmem(table_floats(6, nlam)).total; }
+// Three batches a sub-partition where the slots' state fits beside the filter
+// table, else two (tables of more than about 3,000 points).
+constexpr size_t kWsSmemMax = 227 * 1024;
+static bool ws_three(int nlam) {
+  return WsSmem<kWsBatches>(table_floats(6, nlam)).total <= kWsSmemMax;
+}
 
-cudaError_t invert_ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem) {
-  const size_t sm = invert_ws_smem_bytes(nlam);
-  cudaError_t e = cudaFuncSetAttribute(invert_ws_kernel<6>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+template <int NB>
+static cudaError_t ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem) {
+  auto kern = invert_ws_kernel<6, NB>;
+  const size_t sm = WsSmem<NB>(table_floats(6, nlam)).total;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   nsm = sm_budget(nsm);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, invert_ws_kernel<6>, kWsThreadsN, sm);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kWsThreadsN, sm);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorLaunchOutOfResources;
   // setmaxnreg moves registers within the CTA's launch allocation: the
-  // producers' raise waits for registers the consumers' drop frees, so the
-  // split must fit the registers the kernel is launched with
+  // producers' raise waits for registers the others' drop frees, so the split
+  // must fit the registers the kernel is launched with
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, invert_ws_kernel<6>);
+  e = cudaFuncGetAttributes(&fa, kern);
   if (e != cudaSuccess) return e;
+  // (and setmaxnreg.dec may only go down from the launch's count)
   if ((int64_t)fa.numRegs * kWsThreadsN <
-      (int64_t)32 * (4 * kWsProdRegs + kWsBatches * kWsConsRegs))
+          (int64_t)32 * kWsGroups * (kProdRegs + kAccRegs<NB> + kSolveRegs<NB>) ||
+      fa.numRegs > kProdRegs || fa.numRegs < kAccRegs<NB> || fa.numRegs < kSolveRegs<NB>)
     return cudaErrorInvalidConfiguration;
   int64_t g = nsm;  // one CTA per SM (it holds all of the SM's tensor memory)
-  const int64_t need = (npix + kWsSlotsN - 1) / kWsSlotsN;
+  const int64_t need = (npix + 31) / 32;
   if (need < g) g = need;
   if (g < 1) g = 1;
   *grid = (int)g;
   *smem = sm;
-  *nslots = g * kWsSlotsN;
+  *nslots = g * kWsSlots<NB>;
   return cudaSuccess;
 }
 
+cudaError_t invert_ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem) {
+  return ws_three(nlam) ? ws_slots<kWsBatches>(nlam, npix, nslots, grid, smem)
+                        : ws_slots<2>(nlam, npix, nslots, grid, smem);
+}
+
 cudaError_t launch_invert_ws(const InvertArgs& a, int grid, size_t smem, cudaStream_t s) {
-  invert_ws_kernel<6><<<grid, kWsThreadsN, smem, s>>>(a);
+  // batches of a sub-partition: fewer when the map does not fill them, so
+  // that its pixels spread over all SMs
+  const int64_t per = (int64_t)grid * kWsGroups * 32;
+  const int64_t want = (a.npix + per - 1) / per;
+  const int most = ws_three(a.nlam) ? kWsBatches : 2;
+  const int nb = want < 1 ? 1 : (want > most ? most : (int)want);
+  if (most == kWsBatches)
+    invert_ws_kernel<6, kWsBatches><<<grid, kWsThreadsN, smem, s>>>(a, nb);
+  else
+    invert_ws_kernel<6, 2><<<grid, kWsThreadsN, smem, s>>>(a, nb);
   return cudaGetLastError();
 }
 

