@@ -4,20 +4,26 @@
 // register accumulators (rows x Stokes x filters per thread) cannot hold the
 // whole convolution.  One pixel per warp:
 //   1. the fine grid is walked in chunks of 64 points; each lane evaluates
-//      two points (synthesis and, for the inversion, the six Jacobian rows
-//      of Secs. 3-4, the same per-point arithmetic as the filter kernels)
-//      into a per-warp shared-memory buffer;
-//   2. the samples whose instrument band (at most 32 points) meets the chunk
-//      are spread over the lanes, which add the chunk's points to per-warp
-//      shared accumulators with float4 reads of the transposed chunk;
+//      two points, packed (synthesis and, for the inversion, the six Jacobian
+//      rows of Secs. 3-4, the same per-point arithmetic as the filter
+//      kernels);
+//   2. the instrument profiles are applied.  In the inversion a lane owns one
+//      of the 28 rows; where the samples' bands start one group of four points
+//      after another (a uniform grid), it slides over the groups with the up
+//      to eight samples that meet the current one in registers, each loaded
+//      row value serving all of them.  Other instruments spread the samples
+//      that meet a chunk over the lanes.  The synthesis, with four rows,
+//      spreads the samples over the lanes too, over the whole grid at once;
 //   3. the inversion forms chi2 (Eq. 1; compensated FP32 partial sums,
 //      combined and compared in FP64) and, after an accepted step, J^T W J
 //      and J^T W r, reduced across the warp;
 //   4. the FP64 damped solve (Eqs. 4-5) runs spread over the warp's lanes;
 //      the covariance is left to the batched covariance kernel.
 // The instrument table is compacted on the device into bands (first point,
-// length, weights) and staged in shared memory with one TMA bulk copy.
+// length, weights) and, where they are regular, windows (the weights of the
+// eight groups from a sample's first one), staged in shared memory by TMA.
 #include "common.cuh"
+#include "me_pair.cuh"
 #include "solve.cuh"
 
 namespace vfisv {
@@ -27,24 +33,42 @@ constexpr int kWBand = 32;           // fine points per instrument profile
 constexpr int kWMaxLam = 1024;       // fine grid points
 constexpr int kWChunk = 64;          // fine points per chunk: two per lane
 constexpr int kWMaxChunks = kWMaxLam / kWChunk;
-constexpr int kWWarps = 4;           // pixels in flight per CTA
+constexpr int kWWarps = 9;           // pixels in flight per CTA at most
 constexpr int kWBand4 = kWBand + 4;  // a band starting on a multiple of 4, padded to 4
-constexpr int kWBandStride = kWBand4 + 4;  // [lo4, n4, tau, pad, w[36]] per sample
+constexpr int kWBandStride = kWBand4 + 4;  // [lo4, n4, pad, pad, w[36]] per sample
+constexpr int kWWin = 8;             // groups of four points a window holds
+constexpr int kWWinStride = 4 * kWWin;
 
-// Compacted table: bands [nf][kWBandStride], the active sample range of each
-// chunk [kWMaxChunks][2] (int), then the fine grid x[nlam]; padded to a
-// multiple of 4 floats (16-byte TMA size).
-__host__ __device__ inline int wide_chunks_at(int nf) { return nf * kWBandStride; }
-__host__ __device__ inline int wide_x_at(int nf) { return nf * kWBandStride + 2 * kWMaxChunks; }
+// Compacted table, in 16-byte pieces: header [window groups in use (0: not
+// regular), first group of sample 0's window, 0, 0] (int); tau[nf]; the fine
+// grid x[nlam]; windows, row sg + 7 the weights of the sample whose window
+// starts with group sg (sg from -7 to the last group; zeros where there is
+// none); bands [nf][kWBandStride]; the active sample range of each chunk
+// [kWMaxChunks][2] (int).
+__host__ __device__ inline int up4(int n) { return (n + 3) & ~3; }
+__host__ __device__ inline int wide_groups(int nlam) { return (nlam + 3) / 4; }
+__host__ __device__ inline int wide_x_at(int nf) { return 4 + up4(nf); }
+__host__ __device__ inline int wide_common(int nf, int nlam) { return wide_x_at(nf) + up4(nlam); }
+// (windows past the last group up to a whole half chunk of eight)
+__host__ __device__ inline int wide_groups8(int nlam) { return (nlam + 31) / 32 * 8; }
+__host__ __device__ inline int wide_win_floats(int nlam) {
+  return (wide_groups8(nlam) + kWWin - 1) * kWWinStride;
+}
+__host__ __device__ inline int wide_band_floats(int nf) {
+  return nf * kWBandStride + 2 * kWMaxChunks;
+}
 __host__ __device__ inline int wide_table_floats(int nf, int nlam) {
-  return (wide_x_at(nf) + nlam + 3) & ~3;
+  return wide_common(nf, nlam) + wide_win_floats(nlam) + wide_band_floats(nf);
 }
 
 __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
                                  const float* __restrict__ wl, int nlam,
                                  float* __restrict__ table, int* __restrict__ err) {
   __shared__ int slo[kWMaxF], shi[kWMaxF];
+  __shared__ int start, width;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* win = table + wide_common(nf, nlam);
+  float* bands = win + wide_win_floats(nlam);
   for (int k = warp; k < nf; k += blockDim.x >> 5) {
     const float* row = filters + (size_t)k * nlam;
     // first and last non-zero point; tau in a fixed order (lane-strided
@@ -70,12 +94,12 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
     // length is padded to a multiple of 4 with the zeros around it
     const int lo4 = (n > 0) ? (lo & ~3) : 0;
     const int n4 = (n > 0 && n <= kWBand) ? ((hi - lo4 + 1) + 3) & ~3 : 0;
-    float* b = table + (size_t)k * kWBandStride;
+    float* b = bands + (size_t)k * kWBandStride;
     if (lane == 0) {
       b[0] = __int_as_float(lo4);
       b[1] = __int_as_float(n4);
-      b[2] = s;
-      b[3] = 0.0f;
+      b[2] = b[3] = 0.0f;
+      table[4 + k] = s;  // tau
       slo[k] = lo4;
       shi[k] = lo4 + n4;  // exclusive
     }
@@ -83,8 +107,41 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
       b[4 + t] = (t < n4 && lo4 + t < nlam) ? row[lo4 + t] : 0.0f;
   }
   __syncthreads();
+  // regular bands: sample k's within the window of groups k + start, k +
+  // start + width - 1, for every sample
+  if (warp == 0) {
+    int g0 = 1 << 20, g1 = -(1 << 20);
+    for (int k = lane; k < nf; k += 32)
+      if (shi[k] > slo[k]) g0 = min(g0, slo[k] / 4 - k);
+    for (int o = 16; o > 0; o >>= 1) g0 = min(g0, __shfl_xor_sync(0xffffffffu, g0, o));
+    for (int k = lane; k < nf; k += 32)
+      if (shi[k] > slo[k]) g1 = max(g1, shi[k] / 4 - k);
+    for (int o = 16; o > 0; o >>= 1) g1 = max(g1, __shfl_xor_sync(0xffffffffu, g1, o));
+    if (lane == 0) {
+      // (every sample's window meets the grid: kernels for 7 and 8 groups)
+      const bool ok = g1 > g0 && g1 - g0 <= kWWin &&
+                      g0 > (g1 - g0 < kWWin ? -(kWWin - 1) : -kWWin) &&
+                      g0 + nf <= wide_groups(nlam);
+      start = g0;
+      width = ok ? g1 - g0 : 0;
+      int* h = reinterpret_cast<int*>(table);
+      h[0] = width;
+      h[1] = start;
+      h[2] = h[3] = 0;
+    }
+  }
+  __syncthreads();
+  if (width)
+    for (int t = threadIdx.x; t < wide_win_floats(nlam); t += blockDim.x) {
+      const int sg = t / kWWinStride - (kWWin - 1), k = sg - start;
+      const int i = 4 * sg + t % kWWinStride;  // fine point of this weight
+      float w = 0.0f;
+      if (k >= 0 && k < nf && i >= slo[k] && i < shi[k] && i < nlam)
+        w = filters[(size_t)k * nlam + i];
+      win[t] = w;
+    }
   // samples whose band meets each chunk: [first, last] (their hull)
-  int* ch = reinterpret_cast<int*>(table + wide_chunks_at(nf));
+  int* ch = reinterpret_cast<int*>(bands + nf * kWBandStride);
   for (int c = warp; c < kWMaxChunks; c += blockDim.x >> 5) {
     const int c0 = c * kWChunk, c1 = c0 + kWChunk;
     int kf = 1 << 30, kl = -1;
@@ -102,72 +159,176 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
       ch[2 * c + 1] = kl;
     }
   }
-  for (int i = threadIdx.x; i < nlam; i += blockDim.x) table[wide_x_at(nf) + i] = wl[i];
-  const int tot = wide_table_floats(nf, nlam);
-  for (int i = wide_x_at(nf) + nlam + threadIdx.x; i < tot; i += blockDim.x) table[i] = 0.0f;
+  for (int i = threadIdx.x; i < up4(nlam); i += blockDim.x)
+    table[wide_x_at(nf) + i] = i < nlam ? wl[i] : 0.0f;
+  for (int k = nf + threadIdx.x; k < up4(nf); k += blockDim.x) table[4 + k] = 0.0f;
 }
 
-// Filtered rows of one pixel into the warp's shared accumulators
-// accs[k * P + v], P = 4 R + 1, for every sample k (rows r: Stokes, then
-// with DERIV the six Jacobian rows before their per-pixel scale factors;
-// v = 4 r + Stokes).  vbuf holds one chunk transposed, [4 R][kWChunk].
-template <bool DERIV>
-__device__ __forceinline__ void wide_pass(const Weideman& W, const PixK& P, const float* tab,
-                                          int nf, int nlam, float* vbuf, float* accs, int lane) {
-  constexpr int R = DERIV ? kRows : 1;
-  constexpr int NV = 4 * R, PA = NV + 1;
-  for (int t = lane; t < nf * PA; t += 32) accs[t] = 0.0f;
-  const float* xg = tab + wide_x_at(nf);
-  const int* ch = reinterpret_cast<const int*>(tab + wide_chunks_at(nf));
+// The inversion's buffer of a warp: one chunk of the 28 rows (row stride 68:
+// the lanes' 16-byte reads of their rows meet different banks).
+constexpr int kWRows = 4 * kRows;
+constexpr int kWRowStride = kWChunk + 4;
+constexpr int kWBuf = kWRows * kWRowStride;
+// rows of the accumulators: an odd stride, for lanes owning rows and lanes
+// owning samples alike
+__host__ __device__ inline int wide_acc_stride(int nf) { return nf | 1; }
+
+// Puts the 28 values of two points (columns i, i + 1 of the buffer) there.
+struct WidePut {
+  float* col;
+  f2 iD;
+  __device__ __forceinline__ void put(int v, f2 x) {
+    *reinterpret_cast<unsigned long long*>(col + v * kWRowStride) = x.v;
+  }
+  __device__ __forceinline__ void unit(f2 yI, f2 yQ, f2 yU, f2 yV) {
+    put(0, yI);
+    put(1, yQ);
+    put(2, yU);
+    put(3, yV);
+  }
+  __device__ __forceinline__ void scale(f2 d) { iD = d; }
+  __device__ __forceinline__ void rows(int S, f2 vB, f2 vG, f2 vE, f2 vD, f2 vA, f2 vV) {
+    put(4 * kRowB + S, f2_mul(iD, vB));
+    put(4 * kRowG + S, f2_mul(iD, vG));
+    put(4 * kRowE + S, f2_mul(iD, vE));
+    put(4 * kRowD + S, f2_mul(iD, vD));
+    put(4 * kRowA + S, f2_mul(iD, vA));
+    put(4 * kRowV + S, f2_mul(iD, vV));
+  }
+};
+
+// The rows of the chunk at c0 into the buffer, two points a lane; zeros past
+// the grid.
+__device__ __forceinline__ void wide_chunk(const Weideman& W, const PixK& P, const float* xg,
+                                           int c0, int nlam, float* buf, int lane) {
   __syncwarp();
+  const int i = c0 + 2 * lane;
+  WidePut put{buf + 2 * lane, {}};
+  lambda_pair<true>(W, P, f2_pack(xg[min(i, nlam - 1)], xg[min(i + 1, nlam - 1)]), put);
+  if (c0 + kWChunk > nlam) {
+#pragma unroll 1
+    for (int v = 0; v < kWRows; ++v) {
+      float* row = buf + v * kWRowStride + 2 * lane;
+      if (i >= nlam) row[0] = 0.0f;
+      if (i + 1 >= nlam) row[1] = 0.0f;
+    }
+  }
+  __syncwarp();
+}
+
+// Filtered rows of one pixel into accs[v * wide_acc_stride + k], v = 4 r +
+// Stokes (row r: Stokes, then the six Jacobian rows before their per-pixel
+// scale factors), for every sample k.  A sample's sum is formed chunk by
+// chunk of 64 points, a chunk's part first.
+//
+// With windows of WD groups: lane v slides over the groups of its row.  The
+// sample whose window starts with group sg sits in slot sg mod 8 of a[] and
+// tot[] (static: a half chunk is eight groups).  A group of the row is loaded
+// once for the WD samples that meet it, their weights are broadcasts: 40
+// instructions a group, 4.5 k a pass against 10 k with a sample a lane, 28
+// loads of four conflict-free rows for its 112 sums and a third of the lanes
+// idle.  Instruction fetch bounds the kernel now (about one stall an issue:
+// warps at different places of 20 KB of loop); rolling the pass' loops to
+// half the code cost more instructions than it saved (43.2 -> 48.0 ms).
+template <int WD>
+__device__ __forceinline__ void wide_pass_windows(const Weideman& W, const PixK& P,
+                                                  const float* xg, const float* win, int g0,
+                                                  int nf, int nlam, float* buf, float* accs,
+                                                  int lane) {
+  const int v = min(lane, kWRows - 1);  // the last lanes follow along
+  const int G = wide_groups8(nlam), AS = wide_acc_stride(nf);
+  float* out = accs + v * AS;
+  float a[kWWin], tot[kWWin];
+#pragma unroll
+  for (int u = 0; u < kWWin; ++u) a[u] = tot[u] = 0.0f;
+  const float* wp = win + (kWWin - 1) * kWWinStride;  // window row of the current group
+#pragma unroll 1
+  for (int c0 = 0; c0 < nlam; c0 += kWChunk) {
+    wide_chunk(W, P, xg, c0, nlam, buf, lane);
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      const int gb = c0 / 4 + half * kWWin;  // first group
+      if (gb >= G) break;
+      const float* xb = buf + v * kWRowStride + 4 * kWWin * half;
+      // (the block's results are stored behind it, so that nothing keeps the
+      // next groups' loads from going ahead of the sums)
+      float r[kWWin];
+#pragma unroll
+      for (int u = 0; u < kWWin; ++u) {
+        const float4 x = *reinterpret_cast<const float4*>(xb + 4 * u);
+        a[u] = tot[u] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < WD; ++i) {
+          const float4 w =
+              *reinterpret_cast<const float4*>(wp + u * kWWinStride - i * (kWWinStride - 4));
+          float& s = a[(u - i) & (kWWin - 1)];
+          s = fmaf(w.x, x.x, fmaf(w.y, x.y, fmaf(w.z, x.z, fmaf(w.w, x.w, s))));
+        }
+        r[u] = tot[(u - WD + 1) & (kWWin - 1)] + a[(u - WD + 1) & (kWWin - 1)];
+      }
+      wp += kWWin * kWWinStride;
+      const int k0 = gb - (WD - 1) - g0;  // the sample of r[0]
+      if (lane < kWRows)
+#pragma unroll
+        for (int u = 0; u < kWWin; ++u)
+          if (k0 + u >= 0 && k0 + u < nf) out[k0 + u] = r[u];
+    }
+#pragma unroll
+    for (int u = 0; u < kWWin; ++u) {
+      tot[u] += a[u];
+      a[u] = 0.0f;
+    }
+  }
+  // windows that reach past the last group
+#pragma unroll
+  for (int u = 0; u < kWWin; ++u) {
+    // the last group that started slot u
+    const int sg = G - 1 - ((G - 1 - u) & (kWWin - 1));
+    const int k = sg - g0;
+    if (sg > G - WD && lane < kWRows && k >= 0 && k < nf) out[k] = tot[u] + a[u];
+  }
+  __syncwarp();
+}
+
+// Any bands: the samples that meet a chunk are spread over the lanes.
+__device__ __noinline__ void wide_pass_bands(const Weideman& W, const PixK& P, const float* xg,
+                                             const float* bands, int nf, int nlam, float* buf,
+                                             float* accs, int lane) {
+  const int AS = wide_acc_stride(nf);
+  for (int t = lane; t < kWRows * AS; t += 32) accs[t] = 0.0f;
+  const int* ch = reinterpret_cast<const int*>(bands + nf * kWBandStride);
 #pragma unroll 1
   for (int c0 = 0, c = 0; c0 < nlam; c0 += kWChunk, ++c) {
-#pragma unroll 1
-    for (int t = 0; t < 2; ++t) {
-      const int li = lane + 32 * t, i = c0 + li;
-      float v[R][4][1];
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) v[r][s][0] = 0.0f;
-      if (i < nlam) {
-        const float one[1] = {1.0f};
-        lambda_step<1, DERIV>(W, P, xg[i], one, v);
-      }
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) vbuf[(r * 4 + s) * kWChunk + li] = v[r][s][0];
-    }
-    __syncwarp();
+    wide_chunk(W, P, xg, c0, nlam, buf, lane);
     const int c1 = min(c0 + kWChunk, nlam);
     const int kf = ch[2 * c], kl = ch[2 * c + 1];
 #pragma unroll 1
     for (int k = kf + lane; k <= kl; k += 32) {
-      const float* b = tab + k * kWBandStride;
+      const float* b = bands + k * kWBandStride;
       const int lo4 = __float_as_int(b[0]), n4 = __float_as_int(b[1]);
       const int i0 = max(lo4, c0), i1 = min(lo4 + n4, (c1 + 3) & ~3);
       if (i0 >= i1) continue;
-      float a[NV];
+      float a[kWRows];
 #pragma unroll
-      for (int q = 0; q < NV; ++q) a[q] = 0.0f;
+      for (int q = 0; q < kWRows; ++q) a[q] = 0.0f;
 #pragma unroll 1
       for (int i = i0; i < i1; i += 4) {
         const float4 w = *reinterpret_cast<const float4*>(b + 4 + (i - lo4));
         const int col = i - c0;
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const float4 x = *reinterpret_cast<const float4*>(vbuf + q * kWChunk + col);
+        for (int q = 0; q < kWRows; ++q) {
+          const float4 x = *reinterpret_cast<const float4*>(buf + q * kWRowStride + col);
           a[q] = fmaf(w.x, x.x, fmaf(w.y, x.y, fmaf(w.z, x.z, fmaf(w.w, x.w, a[q]))));
         }
       }
-      float* dst = accs + k * PA;
 #pragma unroll
-      for (int q = 0; q < NV; ++q) dst[q] += a[q];
+      for (int q = 0; q < kWRows; ++q) accs[q * AS + k] += a[q];
     }
-    __syncwarp();
   }
+  __syncwarp();
 }
+
+constexpr int kWSynthWarps = 4;       // pixels in flight per CTA of the synthesis
 
 struct WideSynthArgs {
   const float* params;
@@ -180,46 +341,110 @@ struct WideSynthArgs {
   LineK lk;
 };
 
-// Shared memory of a CTA: the table, then per warp the chunk buffer
-// [4R][kWChunk] and the accumulators [nf][4R + 1] (twice for synthesis: the
-// magnetic and the non-magnetic component), then per warp the LM state.
-__host__ __device__ inline int wide_warp_floats(int nf, bool deriv) {
-  const int nv = deriv ? 4 * kRows : 4;
-  const int acc = nf * (nv + 1) * (deriv ? 1 : 2);
-  return ((nv * kWChunk + acc) + 3) & ~3;
+// Shared memory of a warp: the inversion's buffer and accumulators, or the
+// synthesis' four rows over the whole grid.
+__host__ __device__ inline int wide_warp_floats(int nf, int nlam, bool deriv) {
+  return deriv ? kWBuf + up4(kWRows * wide_acc_stride(nf)) : 4 * (up4(nlam) + 4);
 }
 
-__global__ void __launch_bounds__(32 * kWWarps) wide_synth_kernel(WideSynthArgs A) {
+// Unit-S1 Stokes values of one model over the whole grid into rows[s][GS],
+// two points a lane and round, packed; zeros past the grid.
+__device__ __forceinline__ void wide_synth_rows(const Weideman& W, const PixK& P, const float* xg,
+                                                int nlam, int GS, float* rows, int lane) {
+  struct Take {
+    f2 y[4];
+    __device__ __forceinline__ void unit(f2 yI, f2 yQ, f2 yU, f2 yV) {
+      y[0] = yI;
+      y[1] = yQ;
+      y[2] = yU;
+      y[3] = yV;
+    }
+  } out;
+  __syncwarp();
+#pragma unroll 1
+  for (int c0 = 0; c0 < up4(nlam); c0 += 64) {
+    const int i = c0 + 2 * lane;
+    lambda_pair<false>(W, P, f2_pack(xg[min(i, nlam - 1)], xg[min(i + 1, nlam - 1)]), out);
+    if (i < up4(nlam))
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+        *reinterpret_cast<float2*>(rows + s * GS + i) =
+            make_float2(i < nlam ? f2_lo(out.y[s]) : 0.0f, i + 1 < nlam ? f2_hi(out.y[s]) : 0.0f);
+  }
+  __syncwarp();
+}
+
+// Rows 0 .. NR - 1 through sample k's band, chunk by chunk of 64 points.
+template <int NR>
+__device__ __forceinline__ void wide_synth_sample(const float* bands, int k, int nlam, int GS,
+                                                  const float* rows, float (&y)[NR]) {
+  const float* b = bands + k * kWBandStride;
+  const int lo4 = __float_as_int(b[0]), n4 = __float_as_int(b[1]);
+  const int hi = min(lo4 + n4, up4(nlam));
+#pragma unroll
+  for (int s = 0; s < NR; ++s) y[s] = 0.0f;
+#pragma unroll 1
+  for (int i = lo4; i < hi;) {
+    const int end = min(hi, (i / kWChunk + 1) * kWChunk);
+    float a[NR];
+#pragma unroll
+    for (int s = 0; s < NR; ++s) a[s] = 0.0f;
+#pragma unroll 1
+    for (; i < end; i += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(b + 4 + (i - lo4));
+#pragma unroll
+      for (int s = 0; s < NR; ++s) {
+        const float4 x = *reinterpret_cast<const float4*>(rows + s * GS + i);
+        a[s] = fmaf(w.x, x.x, fmaf(w.y, x.y, fmaf(w.z, x.z, fmaf(w.w, x.w, a[s]))));
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < NR; ++s) y[s] += a[s];
+  }
+}
+
+__global__ void __launch_bounds__(32 * kWSynthWarps) wide_synth_kernel(WideSynthArgs A) {
   extern __shared__ __align__(16) float smem[];
-  const int tabf = wide_table_floats(A.nf, A.nlam);
-  const int wf = wide_warp_floats(A.nf, false);
+  const int nf = A.nf, nlam = A.nlam;
+  const int cf = wide_common(nf, nlam), bf = wide_band_floats(nf);
+  const int wf = wide_warp_floats(nf, nlam, false), GS = up4(nlam) + 4;
   float* tab = smem;
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + tabf + kWWarps * wf);
-  if (!tma_load_table(tab, A.table, (uint32_t)(tabf * sizeof(float)), mbar, A.err)) return;
+  float* bands = smem + cf;
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(bands + bf + kWSynthWarps * wf);
+  if (!tma_load_table(tab, A.table, (uint32_t)(cf * sizeof(float)), mbar, A.err)) return;
+  if (!tma_load_table(bands, A.table + cf + wide_win_floats(nlam),
+                      (uint32_t)(bf * sizeof(float)), mbar + 1, A.err))
+    return;
   if (*A.err) return;  // a band wider than the kernel takes
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nf = A.nf;
-  float* vbuf = smem + tabf + warp * wf;
-  float* acc = vbuf + 4 * kWChunk;
-  float* accn = acc + nf * 5;
-  for (int64_t pix = (int64_t)blockIdx.x * kWWarps + warp; pix < A.npix;
-       pix += (int64_t)gridDim.x * kWWarps) {
+  float* rows = bands + bf + warp * wf;
+  const float* xg = tab + wide_x_at(nf);
+  for (int64_t pix = (int64_t)blockIdx.x * kWSynthWarps + warp; pix < A.npix;
+       pix += (int64_t)gridDim.x * kWSynthWarps) {
     const float* p = A.params + pix * 10;
     const float B = p[0], gam = p[1], psi = p[2], eta0 = p[3], dld = p[4], dmp = p[5],
                 v = p[6], S0 = p[7], S1 = p[8], alpha = p[9];
-    wide_pass<false>(A.W, make_pixk(A.lk, B, gam, eta0, dld, dmp, v), tab, nf, A.nlam, vbuf,
-                     acc, lane);
-    if (alpha != 1.0f)  // non-magnetic component: the same line with B = 0
-      wide_pass<false>(A.W, make_pixk(A.lk, 0.0f, gam, eta0, dld, dmp, v), tab, nf, A.nlam,
-                       vbuf, accn, lane);
     float c2, s2;
     sincosf(2.0f * psi * kDeg, &s2, &c2);
     const float mus1 = A.lk.mu * S1;
     float* out = A.stokes + pix * 4 * nf;
+    // the non-magnetic component first (the same line with B = 0): its Stokes
+    // I waits in the output
+    if (alpha != 1.0f) {
+      wide_synth_rows(A.W, make_pixk(A.lk, 0.0f, gam, eta0, dld, dmp, v), xg, nlam, GS, rows,
+                      lane);
+      for (int k = lane; k < nf; k += 32) {
+        float y[1];
+        wide_synth_sample<1>(bands, k, nlam, GS, rows, y);
+        out[k] = y[0];
+      }
+    }
+    wide_synth_rows(A.W, make_pixk(A.lk, B, gam, eta0, dld, dmp, v), xg, nlam, GS, rows, lane);
     for (int k = lane; k < nf; k += 32) {
-      const float tau = tab[k * kWBandStride + 2];
-      const float* a = acc + k * 5;
-      const float In = (alpha != 1.0f) ? accn[k * 5] : 0.0f;
+      float a[4];
+      wide_synth_sample<4>(bands, k, nlam, GS, rows, a);
+      const float tau = tab[4 + k];
+      const float In = (alpha != 1.0f) ? out[k] : 0.0f;
       const float yI = alpha * a[0] + (1.0f - alpha) * In;
       const float yQ = alpha * a[1], yU = alpha * a[2], yV = alpha * a[3];
       out[k] = fmaf(S0, tau, mus1 * yI);
@@ -227,7 +452,6 @@ __global__ void __launch_bounds__(32 * kWWarps) wide_synth_kernel(WideSynthArgs 
       out[2 * nf + k] = mus1 * fmaf(s2, yQ, c2 * yU);
       out[3 * nf + k] = mus1 * yV;
     }
-    __syncwarp();
   }
 }
 
@@ -352,19 +576,35 @@ struct WideWarpState {
   int it;
 };
 
+// windows or bands, whichever the instrument has
+__host__ __device__ inline int wide_part_floats(int nf, int nlam) {
+  return max(wide_win_floats(nlam), wide_band_floats(nf));
+}
+
 __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs A, int nf) {
   extern __shared__ __align__(16) float smem[];
-  const int tabf = wide_table_floats(nf, A.nlam);
-  const int wf = wide_warp_floats(nf, true);
+  const int nlam = A.nlam, nwarps = blockDim.x >> 5;
+  const int cf = wide_common(nf, nlam);
+  const int pf = wide_part_floats(nf, nlam);
+  const int wf = wide_warp_floats(nf, nlam, true);
   float* tab = smem;
-  WideWarpState* states = reinterpret_cast<WideWarpState*>(smem + tabf + kWWarps * wf);
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(states + kWWarps);
-  if (!tma_load_table(tab, A.table, (uint32_t)(tabf * sizeof(float)), mbar, A.err)) return;
+  float* part = smem + cf;  // windows or bands
+  WideWarpState* states = reinterpret_cast<WideWarpState*>(part + pf + nwarps * wf);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(states + nwarps);
+  if (!tma_load_table(tab, A.table, (uint32_t)(cf * sizeof(float)), mbar, A.err)) return;
   if (*A.err) return;
+  const int width = reinterpret_cast<const int*>(tab)[0];
+  const int start = reinterpret_cast<const int*>(tab)[1];
+  if (!tma_load_table(part, A.table + cf + (width ? 0 : wide_win_floats(nlam)),
+                      (uint32_t)((width ? wide_win_floats(nlam) : wide_band_floats(nf)) *
+                                 sizeof(float)),
+                      mbar + 1, A.err))
+    return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* vbuf = smem + tabf + warp * wf;
-  float* accs = vbuf + 4 * kRows * kWChunk;
-  constexpr int PA = 4 * kRows + 1;
+  float* buf = part + pf + warp * wf;
+  float* accs = buf + kWBuf;
+  const int AS = wide_acc_stride(nf);
+  const float* taus = tab + 4;
   WideWarpState& S = states[warp];
   const int nobs = 4 * nf;
   const int dof = nobs - A.nfree;
@@ -438,15 +678,14 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
       // ---- damped step (Eqs. 4-5), FP64 over the warp ----
       const double eps = S.eps;
       const bool ok = warp_damped_step(S.A, A.free_mask, eps, lane, S.delta);
+      if (!ok && lane == 0) damped_step_fp64(S.A, 1, A.free_mask, eps, S.delta);  // eigen fallback
+      __syncwarp();
+      // parameter j on lane j: the FP64 sums side by side
+      if (lane < kNP) S.Mt[lane] = (float)((double)S.M[lane] + S.delta[lane]);
+      __syncwarp();
       if (lane == 0) {
-        double d[kNP];
-        if (ok) {
-          for (int j = 0; j < kNP; ++j) d[j] = S.delta[j];
-        } else {
-          damped_step_fp64(S.A, 1, A.free_mask, eps, d);  // with the eigen fallback
-        }
         float Mt[10];
-        for (int j = 0; j < kNP; ++j) Mt[j] = (float)((double)S.M[j] + d[j]);
+        for (int j = 0; j < kNP; ++j) Mt[j] = S.Mt[j];
         Mt[9] = 1.0f;
         apply_bounds(Mt);
         for (int j = 0; j < 10; ++j) S.Mt[j] = Mt[j];
@@ -458,8 +697,16 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
     float Mt[10];
 #pragma unroll
     for (int j = 0; j < 10; ++j) Mt[j] = S.Mt[j];
-    wide_pass<true>(A.W, make_pixk(A.lk, Mt[0], Mt[1], Mt[3], Mt[4], Mt[5], Mt[6]), tab, nf,
-                    A.nlam, vbuf, accs, lane);
+    {
+      const PixK P = make_pixk(A.lk, Mt[0], Mt[1], Mt[3], Mt[4], Mt[5], Mt[6]);
+      const float* xg = tab + wide_x_at(nf);
+      if (width == kWWin)
+        wide_pass_windows<kWWin>(A.W, P, xg, part, start, nf, nlam, buf, accs, lane);
+      else if (width)
+        wide_pass_windows<kWWin - 1>(A.W, P, xg, part, start, nf, nlam, buf, accs, lane);
+      else
+        wide_pass_bands(A.W, P, xg, part, nf, nlam, buf, accs, lane);
+    }
     const long long pix = S.pix;
     const float* o = A.obs + pix * nobs;
     const float* wv = weight_row(A, pix, nobs);
@@ -475,11 +722,11 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
       float qs = 0.0f, qc = 0.0f;
 #pragma unroll 1
       for (int k = lane; k < nf; k += 32) {
-        const float tau = tab[k * kWBandStride + 2];
-        const float* a = accs + k * PA;
-        const float q0 = a[1], u0 = a[2];
+        const float tau = taus[k];
+        const float* a = accs + k;
+        const float q0 = a[AS], u0 = a[2 * AS];
         const float syn[4] = {fmaf(s0, tau, mus1 * a[0]), mus1 * fmaf(c2p, q0, -s2p * u0),
-                              mus1 * fmaf(s2p, q0, c2p * u0), mus1 * a[3]};
+                              mus1 * fmaf(s2p, q0, c2p * u0), mus1 * a[3 * AS]};
 #pragma unroll
         for (int st = 0; st < 4; ++st) {
           const float r = o[st * nf + k] - syn[st];
@@ -538,9 +785,9 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
       for (int i = 0; i < kNP; ++i) g[i] = 0.0f;
 #pragma unroll 1
       for (int k = lane; k < nf; k += 32) {
-        const float tau = tab[k * kWBandStride + 2];
-        const float* a = accs + k * PA;
-        const float q0 = a[1], u0 = a[2];
+        const float tau = taus[k];
+        const float* a = accs + k;
+        const float q0 = a[AS], u0 = a[2 * AS];
         const float Qk = mus1 * fmaf(c2p, q0, -s2p * u0);
         const float Uk = mus1 * fmaf(s2p, q0, c2p * u0);
 #pragma unroll 1
@@ -554,10 +801,10 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
           for (int pp = 0; pp < kNP; ++pp)
             if (rowOf[pp] >= 0)
               J[pp] = (mus1 * Rs.s[rowOf[pp]]) *
-                      fmaf(cA, a[rowOf[pp] * 4 + sa], cB * a[rowOf[pp] * 4 + sb]);
+                      fmaf(cA, a[(rowOf[pp] * 4 + sa) * AS], cB * a[(rowOf[pp] * 4 + sb) * AS]);
           J[2] = (st == 1) ? -2.0f * kDeg * Uk : (st == 2 ? 2.0f * kDeg * Qk : 0.0f);
           J[7] = (st == 0) ? tau : 0.0f;
-          const float lin = fmaf(cA, a[sa], cB * a[sb]);
+          const float lin = fmaf(cA, a[sa * AS], cB * a[sb * AS]);
           J[8] = mu * lin;
           const float sv = (st == 0) ? fmaf(s0, tau, mus1 * lin) : mus1 * lin;
           const float ww = wv[st * nf + k];
@@ -571,16 +818,27 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
           }
         }
       }
+      // sums over the lanes: the butterfly of warp_sum(), halving the values a
+      // lane carries at every step (54 exchanges instead of 270); lane l ends
+      // with elements l and l + 32
+      float v[64];
 #pragma unroll
-      for (int i = 0; i < kNPk; ++i) am[i] = warp_sum(am[i]);
+      for (int i = 0; i < 64; ++i)
+        v[i] = (i < kNPk) ? am[i] : (i < kNPk + kNP ? g[i < kNPk ? 0 : i - kNPk] : 0.0f);
 #pragma unroll
-      for (int i = 0; i < kNP; ++i) g[i] = warp_sum(g[i]);
+      for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+          if (!(i & (32 - o))) {  // elements i (kept by the lower lanes) and i + o
+            const float keep = up ? v[i + o] : v[i], give = up ? v[i] : v[i + o];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+      }
       __syncwarp();
-      if (lane == 0) {  // every lane holds the totals
-#pragma unroll
-        for (int i = 0; i < kNPk; ++i) S.A[i] = am[i];
-#pragma unroll
-        for (int i = 0; i < kNP; ++i) S.A[kNPk + i] = g[i];
+      S.A[lane] = v[0];
+      if (lane + 32 < kNPk + kNP) S.A[lane + 32] = v[32];
+      if (lane == 0) {
         for (int j = 0; j < 10; ++j) S.M[j] = Mt[j];
         S.chi2b = c2;
       }
@@ -620,15 +878,15 @@ __global__ void __launch_bounds__(32 * kWWarps, 1) wide_invert_kernel(InvertArgs
 
 size_t wide_table_bytes(int nf, int nlam) { return (size_t)wide_table_floats(nf, nlam) * 4; }
 
-static size_t wide_smem(int nf, int nlam, bool invert) {
-  size_t b = (size_t)(wide_table_floats(nf, nlam) + kWWarps * wide_warp_floats(nf, invert)) * 4;
-  if (invert) b += kWWarps * sizeof(WideWarpState);
+static size_t wide_smem(int nf, int nlam, bool invert, int warps) {
+  const int part = invert ? wide_part_floats(nf, nlam) : wide_band_floats(nf);
+  size_t b = (size_t)(wide_common(nf, nlam) + part + warps * wide_warp_floats(nf, nlam, invert)) * 4;
+  if (invert) b += warps * sizeof(WideWarpState);
   return ((b + 15) & ~(size_t)15) + 16;
 }
 
 bool wide_supported(int nf, int nlam) {
-  return nf >= 1 && nf <= kWMaxF && nlam >= 1 && nlam <= kWMaxLam &&
-         wide_smem(nf, nlam, true) <= 227 * 1024;
+  return nf >= 1 && nf <= kWMaxF && nlam >= 1 && nlam <= kWMaxLam;
 }
 
 cudaError_t launch_wide_pack(const float* filters, int nf, const float* wl, int nlam,
@@ -639,39 +897,49 @@ cudaError_t launch_wide_pack(const float* filters, int nf, const float* wl, int 
   return cudaGetLastError();
 }
 
-static int wide_grid(const void* kern, size_t smem, int64_t npix) {
+cudaError_t launch_wide_synth(const float* params, int64_t npix, const float* table, int nf,
+                              int nlam, float* stokes, int* err, const Weideman& W,
+                              const LineK& lk, cudaStream_t s) {
+  const size_t smem = wide_smem(nf, nlam, false, kWSynthWarps);
+  cudaError_t e = cudaFuncSetAttribute(wide_synth_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   nsm = sm_budget(nsm);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * kWWarps, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, wide_synth_kernel, 32 * kWSynthWarps, smem);
   if (per < 1) per = 1;
   int64_t g = (int64_t)nsm * per;
-  const int64_t need = (npix + kWWarps - 1) / kWWarps;
+  const int64_t need = (npix + kWSynthWarps - 1) / kWSynthWarps;
   if (need < g) g = need;
-  return (int)(g < 1 ? 1 : g);
-}
-
-cudaError_t launch_wide_synth(const float* params, int64_t npix, const float* table, int nf,
-                              int nlam, float* stokes, int* err, const Weideman& W,
-                              const LineK& lk, cudaStream_t s) {
-  const size_t smem = wide_smem(nf, nlam, false);
-  cudaError_t e = cudaFuncSetAttribute(wide_synth_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  if (g < 1) g = 1;
   WideSynthArgs a{params, npix, table, nf, nlam, stokes, err, W, lk};
-  wide_synth_kernel<<<wide_grid((const void*)wide_synth_kernel, smem, npix), 32 * kWWarps, smem,
-                      s>>>(a);
+  wide_synth_kernel<<<(int)g, 32 * kWSynthWarps, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_wide_invert(const InvertArgs& a, int nf, cudaStream_t s) {
-  const size_t smem = wide_smem(nf, a.nlam, true);
+  int dev = 0, nsm = 0, most = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  nsm = sm_budget(nsm);
+  // one CTA per SM, a pixel a warp: as many warps as the shared memory holds
+  // (9 with 112 samples: 65,536 pixels 41.9 ms, with 8 43.2; halving the
+  // chunk's buffer made room for 12, 43.1), fewer when the map does not fill
+  // them, so that its pixels spread over all SMs
+  int64_t warps = (a.npix + nsm - 1) / nsm;
+  if (warps > kWWarps) warps = kWWarps;
+  if (warps < 1) warps = 1;
+  while (warps > 1 && wide_smem(nf, a.nlam, true, (int)warps) > (size_t)most) --warps;
+  const size_t smem = wide_smem(nf, a.nlam, true, (int)warps);
   cudaError_t e = cudaFuncSetAttribute(wide_invert_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  wide_invert_kernel<<<wide_grid((const void*)wide_invert_kernel, smem, a.npix), 32 * kWWarps,
-                       smem, s>>>(a, nf);
+  int64_t g = (a.npix + warps - 1) / warps;
+  if (g > nsm) g = nsm;
+  wide_invert_kernel<<<(int)(g < 1 ? 1 : g), 32 * (int)warps, smem, s>>>(a, nf);
   return cudaGetLastError();
 }
 
