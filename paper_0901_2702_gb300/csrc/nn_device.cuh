@@ -29,6 +29,50 @@ __device__ __forceinline__ float ic_of(const float* o) {
   return fmaxf(ic, 1e-30f);
 }
 
+// mult < n, offset + m < 2n and n < 2^31 keep the product inside 64 bits.
+__device__ __forceinline__ int64_t sample_of(int64_t m, const Perm& p) {
+  return (int64_t)((p.mult * (uint64_t)(p.offset + m) + p.add) % (uint64_t)p.n);
+}
+
+// Training targets of a parameter vector.
+__device__ __forceinline__ void targets(const float* p, float ic, float (&t)[OUT - 1]) {
+  const float g = p[1] * 0.017453292519943295f, ps = p[2] * 0.034906585039886591f;
+  t[0] = p[0];
+  t[1] = cosf(g);
+  t[2] = sinf(ps);
+  t[3] = cosf(ps);
+  t[4] = logf(p[3]);
+  t[5] = p[4];
+  t[6] = p[5];
+  t[7] = p[6];
+  t[8] = p[7] / ic;
+  t[9] = p[8] / ic;
+}
+
+// Loss of a sample (the regression of Sec. 5 plus the confidence output) with
+// outputs y[0..10] and parameters p, and its gradient d = dL/dy for a batch of
+// `rows` samples.
+__device__ __forceinline__ float loss_row(const float* y, const float* p, float ic,
+                                          const float* mean, const float* std, float rows,
+                                          float* d) {
+  float t[OUT - 1];
+  targets(p, ic, t);
+  const float invn = 1.0f / rows;
+  float e[OUT - 1], mse = 0.0f;
+#pragma unroll
+  for (int o = 0; o < OUT - 1; ++o) {
+    const float ts = (t[o] - mean[o]) / std[o];
+    e[o] = y[o] - ts;
+    mse = fmaf(e[o], e[o], mse);
+  }
+  const float c = logf(mse / (OUT - 1) + 1e-4f);
+  const float ec = y[OUT - 1] - c;
+#pragma unroll
+  for (int o = 0; o < OUT - 1; ++o) d[o] = 2.0f * e[o] * invn / (OUT - 1);
+  d[OUT - 1] = 2.0f * ec * invn;
+  return mse * invn / (OUT - 1) + ec * ec * invn;
+}
+
 // Network outputs y[0..10] (standardised, bias included) -> initial model
 // p[0..9]; the inverse of the training targets [B, cos gamma, sin 2psi,
 // cos 2psi, ln eta0, dlambdaD, a, v, S0/Ic, S1/Ic].

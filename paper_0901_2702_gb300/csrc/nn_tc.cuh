@@ -1,9 +1,11 @@
-// The tcgen05 training GEMM (nn_tc.cu) and its operand layout, used by the
-// network's forward and backward passes (nn.cu).
+// The tcgen05 training kernels (nn_tc.cu) and their operand layout, used by
+// the network's training step (nn.cu).
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "nn.cuh"
 
 namespace vfisv {
 namespace nn {
@@ -17,37 +19,38 @@ __host__ __device__ constexpr size_t tl_off(int64_t r, int c, int64_t R) {
          (size_t)((c & 63) >> 3) * 128 + (size_t)(r & 7) * 16 + (size_t)(c & 7) * 2;
 }
 
-// Epilogues of D = A B^T (rows of D = rows of A).
-enum TcEpi : int {
-  EPI_HIDDEN = 0,   // z = D + bias -> Z (FP32, row-major); GELU(z) -> H, HT (BF16, TL)
-  EPI_OUT = 1,      // D + bias (first n_valid columns) -> Z (FP32, row-major)
-  EPI_DX = 2,       // D * GELU'(Zprev) -> H, HT (BF16, TL); H may be null
-  EPI_PARTIAL = 3,  // D of this K split -> P[split][MA][N] (FP32)
-};
+// Padded widths of the training operands: the transposed features (24) have
+// 32 rows, the outputs (11) and their gradient 16; the packed weights' K is a
+// multiple of 64.
+constexpr int XK = 64, XT = 32, YN = 16, DYK = 64;
 
-struct TcGemmArgs {
-  const uint8_t* A;  // TL(MA, K)
-  int64_t MA;        // rows of A (a multiple of 128) = rows of D
-  const uint8_t* B;  // TL(NB, K), NB = N
-  int64_t NB;
-  int K;                  // a multiple of 64
-  int kchunks_per_split;  // 64-wide K-chunks per blockIdx.y
-  const float* bias;
-  int n_valid;
-  float* Z;
-  int64_t ldz;
-  uint8_t* H;   // TL(MA, N)
-  uint8_t* HT;  // TL(N, MA)
-  const float* Zprev;
-  int64_t ldzp;
-  float* P;
+// Forward and backward pass of the rows 0 .. 128 tiles - 1 of a batch, of
+// which the first `rows` are samples and the rest padding.
+struct TrainPassArgs {
+  const float *blob, *obs, *params;
+  Perm perm;
+  int64_t rows;
+  PackedNet P;
+  uint8_t *XT, *HT[3];    // transposed features TL(32, M), activations TL(256, M)
+  uint8_t *dYT, *dZT[3];  // transposed gradients TL(16, M), TL(256, M)
+  float* loss;            // a row's loss (0 on padding), [M]
   int* err;
 };
+cudaError_t train_pass(const TrainPassArgs& a, int64_t tiles, cudaStream_t s);
 
-// D tiles of N in {16, 32, 256} columns; grid mtiles x splits.  Returns
-// cudaErrorInvalidValue for shapes the kernel does not take (K or MA not
-// multiples of 64 / 128, a split without K-chunks, an unsupported N/epilogue).
-cudaError_t tc_gemm(const TcGemmArgs& g, int n, int epi, int mtiles, int splits, cudaStream_t s);
+// Weight and bias gradients, split over the batch: split s takes K-chunks
+// (64 rows) s per .. s per + per - 1 of `chunks`; and the loss of each 256 rows.
+struct TrainDwArgs {
+  const uint8_t *XT, *HT[3], *dYT, *dZT[3];
+  float* wpart[4];  // [splits][256][32: W0^T | 256 | 256 | 16]
+  float* bpart[4];  // [splits][256 | 256 | 256 | 16]
+  const float* loss;
+  float* lossp;
+  int nloss, chunks, per;
+  int* err;
+};
+// cudaErrorInvalidValue unless every split owns at least one chunk.
+cudaError_t train_dw(const TrainDwArgs& a, int splits, cudaStream_t s);
 
 }  // namespace nn
 }  // namespace vfisv
