@@ -77,6 +77,11 @@ constexpr uint32_t kSend = 2 * kOpChunk;          // a CTA's half of it
 constexpr int NSLOT = 4;
 constexpr int KX = XT;                            // features padded to two K = 16 steps
 constexpr int NY = YN;                            // outputs padded
+// columns an epilogue takes at once, in a rolled loop: a CTA runs each layer's
+// code once or thrice, so that unrolling it costs instruction fetches (a step
+// of 8192 samples takes 75.5 us with 8, 1 more with 16, 4 more with 32)
+constexpr int kEpc = 8;
+constexpr int kPassLaunch = kThreads + 32;  // and a warp that loads the weights
 constexpr int kStreamed = 18;  // weight chunks a tile: W0 1, W1 4, W2 4, W3^T 1, W2^T 4, W1^T 4
 
 constexpr uint32_t PM_RING = 0;
@@ -100,6 +105,25 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
+}
+
+// barriers of the computing warps
+__device__ __forceinline__ void compute_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+}
+__device__ __forceinline__ bool compute_sync_or(bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)p), "n"(kThreads)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
 }
 
 // Four transposed 8 x 8 matrices: lane l gives the address of row l % 8 of
@@ -132,7 +156,7 @@ __device__ __forceinline__ void put_transposed(Off off, uint32_t sbo, int groups
   }
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPassLaunch, 1)
     train_pass_kernel(TrainPassArgs a) {
   extern __shared__ uint8_t smem_raw[];
   // (the same offset in both CTAs: dynamic shared memory starts alike)
@@ -152,7 +176,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     for (int i = 0; i < 2 * NSLOT + 4; ++i) bar_init(bar_full + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int i = tid; i < 3 * HID; i += kThreads) {
+  for (int i = tid; i < 3 * HID; i += kPassLaunch) {
     const int l = i / HID;
     bias[i] = a.blob[(l == 0 ? OFF_B0 : l == 1 ? OFF_B1 : OFF_B2) + i % HID];
   }
@@ -168,32 +192,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc_before_sync();
   __syncthreads();
   // the peer's barriers are initialised before anything is sent to it
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
+  cluster_sync();
   tc_after_sync();
   const uint32_t tmem = *tmem_slot;
 
-  // issuer state (thread 0): weight chunks consumed, loaded and landed,
-  // arrivals from the peer, a sticky timeout flag
-  int g_cons = 0, g_load = 0, g_landed = 0, n_half = 0, n_sent = 0;
-  bool ibad = false;
-  auto load_chunk = [&](int g) {
-    const uint8_t* src;
-    if (g < 1) src = a.P.Wt[0];
-    else if (g < 5) src = a.P.Wt[1] + (size_t)(g - 1) * 2 * kHalf;
-    else if (g < 9) src = a.P.Wt[2] + (size_t)(g - 5) * 2 * kHalf;
-    else if (g < 10) src = a.P.Wn[3];
-    else if (g < 14) src = a.P.Wn[2] + (size_t)(g - 10) * 2 * kHalf;
-    else src = a.P.Wn[1] + (size_t)(g - 14) * 2 * kHalf;
-    const uint32_t bar = bar_full + 8 * (g % NSLOT);
-    expect_tx(bar, kHalf);
-    bulk_load(sb + PM_RING + (g % NSLOT) * kHalf, src + rank * kHalf, kHalf, bar);
-  };
-  if (tid == 0) {
-    expect_tx(bar_w3, NY * HID * 2);
-    bulk_load(sb + PM_W3, a.P.Wt[3], NY * HID * 2, bar_w3);
-    for (; g_load < NSLOT - 1; ++g_load) load_chunk(g_load);
+  if (warp == kThreads / 32) {
+    // weight loads: their own warp, so that neither they wait for an issue nor
+    // an issue for a slot
+    if (lane == 0) {
+      expect_tx(bar_w3, NY * HID * 2);
+      bulk_load(sb + PM_W3, a.P.Wt[3], NY * HID * 2, bar_w3);
+      int g = 0;
+      for (; g < kStreamed; ++g) {
+        const int slot = g % NSLOT;
+        const uint8_t* src;
+        if (g < 1) src = a.P.Wt[0];
+        else if (g < 5) src = a.P.Wt[1] + (size_t)(g - 1) * 2 * kHalf;
+        else if (g < 9) src = a.P.Wt[2] + (size_t)(g - 5) * 2 * kHalf;
+        else if (g < 10) src = a.P.Wn[3];
+        else if (g < 14) src = a.P.Wn[2] + (size_t)(g - 10) * 2 * kHalf;
+        else src = a.P.Wn[1] + (size_t)(g - 14) * 2 * kHalf;
+        if (g >= NSLOT && !mbar_wait(bar_empty + 8 * slot, (g / NSLOT - 1) & 1)) break;
+        expect_tx(bar_full + 8 * slot, kHalf);
+        bulk_load(sb + PM_RING + slot * kHalf, src + rank * kHalf, kHalf, bar_full + 8 * slot);
+      }
+      // the copies land, and of a whole stream the tensor cores' last arrivals
+      // come, before the memory is released
+      mbar_wait(bar_w3, 0);
+      for (int i = g > NSLOT ? g - NSLOT : 0; i < g; ++i) {
+        mbar_wait(bar_full + 8 * (i % NSLOT), (i / NSLOT) & 1);
+        if (g == kStreamed) mbar_wait(bar_empty + 8 * (i % NSLOT), (i / NSLOT) & 1);
+      }
+      if (g < kStreamed) atomicExch(a.err, kDevErrNnWait);
+    }
+    __syncwarp();
+    __syncthreads();
+    cluster_sync();
+    return;
   }
+
+  // issuer state (thread 0): weight chunks consumed, arrivals from the peer,
+  // halves sent to it, a sticky timeout flag
+  int g_cons = 0, n_half = 0, n_sent = 0;
+  bool ibad = false;
   constexpr uint32_t kIdescHalf = idesc_bf16(TMR, NH), kIdescOut = idesc_bf16(TMR, NY);
   // MMAs of the next weight chunk: `steps` K = 16 steps of the operand at A
   auto issue_chunk = [&](uint32_t d, uint32_t A, uint32_t sbo, int steps, bool first) {
@@ -203,22 +244,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       ibad = true;
       return;
     }
-    g_landed = g + 1;
     for (int ks = 0; ks < steps; ++ks)
       mma_bf16(d, sdesc(A + ks * 256, 128, sbo),
                sdesc(sb + PM_RING + slot * kHalf + ks * 256, 128, 1024), kIdescHalf,
                !(first && ks == 0));
     mma_commit(bar_empty + 8 * slot);
-    // refill the slot of chunk g - 1 (its MMAs were issued earlier) with g + 3
-    const int gn = g + NSLOT - 1;
-    if (gn < kStreamed) {
-      if (gn >= NSLOT && !mbar_wait(bar_empty + 8 * (gn % NSLOT), (gn / NSLOT - 1) & 1)) {
-        ibad = true;
-      } else {
-        load_chunk(gn);
-        g_load = gn + 1;
-      }
-    }
   };
   // a product over the whole operand in buffer `buf`, whose other half comes
   // from the peer: own K-chunks first would change the order of the sum, so
@@ -235,7 +265,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto sync_mma = [&]() -> bool {
     const bool ok = mbar_wait(bar_mma, mph);
     mph ^= 1;
-    if (__syncthreads_or(!ok || (tid == 0 && ibad))) return false;
+    if (compute_sync_or(!ok || (tid == 0 && ibad))) return false;
     tc_after_sync();
     return true;
   };
@@ -243,21 +273,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int lq = warp & 3, cq = warp >> 2, row = 32 * lq + lane;
   const uint32_t tlane = tmem + ((uint32_t)(32 * lq) << 16);
   const int c0 = (int)rank * NH + 32 * cq;  // this warp's first column
-  // the warp's 32 columns of a new operand (BF16) into buffer `buf`
-  auto put_operand = [&](const float (&h)[32], int buf) {
-    uint8_t* p = sm + PM_H + buf * kOp + (c0 >> 6) * kOpChunk + (row >> 3) * 1024 + (row & 7) * 16 +
-                 ((c0 & 63) >> 3) * 128;
-#pragma unroll
-    for (int j = 0; j < 32; j += 8)
-      *reinterpret_cast<uint4*>(p + (j >> 3) * 128) =
-          make_uint4(pack_bf16x2(h[j], h[j + 1]), pack_bf16x2(h[j + 2], h[j + 3]),
-                     pack_bf16x2(h[j + 4], h[j + 5]), pack_bf16x2(h[j + 6], h[j + 7]));
+  // columns c .. c + 7 of a new operand (BF16) into buffer `buf`
+  auto put_operand = [&](const f2 (&h)[4], int buf, int c) {
+    *reinterpret_cast<uint4*>(sm + PM_H + buf * kOp + (c >> 6) * kOpChunk + (row >> 3) * 1024 +
+                              (row & 7) * 16 + ((c & 63) >> 3) * 128) =
+        make_uint4(pack_bf16x2(f2_lo(h[0]), f2_hi(h[0])), pack_bf16x2(f2_lo(h[1]), f2_hi(h[1])),
+                   pack_bf16x2(f2_lo(h[2]), f2_hi(h[2])), pack_bf16x2(f2_lo(h[3]), f2_hi(h[3])));
+  };
+  // accumulator column pair + bias
+  auto z_pair = [&](float lo, float hi, const float* b) {
+    const float2 bb = *reinterpret_cast<const float2*>(b);
+    return f2_add(f2_pack(lo, hi), f2_pack(bb.x, bb.y));
   };
   // after an epilogue: the CTA's half is in buffer `buf`; sends it to the peer
   auto publish = [&](int buf, bool send) {
     fence_async_smem();
     tc_before_sync();
-    __syncthreads();
+    compute_sync();
     if (send && tid == 0) {
       const uint32_t off = sb + PM_H + buf * kOp + rank * kSend, bar = bar_half + 8 * buf;
       expect_tx(bar, kSend);  // what the peer sends here
@@ -302,7 +334,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           make_uint4(pk[0], pk[1], pk[2], pk[3]);
       fence_async_smem();
       tc_before_sync();
-      __syncthreads();
+      compute_sync();
     }
     // ---- forward: layers 0 to 2 into accumulators 0 to 2 ----
 #pragma unroll 1
@@ -322,11 +354,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                        a.XT, KX, 0, m0, warp, lane);
       if (l > 0) copy_out((l - 1) & 1, a.HT[l - 1]);
       if (!(ok = sync_mma())) break;
-      float v[32];
-      tmem_ld32(tlane + (uint32_t)(l * NH + 32 * cq), v);
+#pragma unroll 1
+      for (int c = 0; c < 32; c += kEpc) {
+        float v[kEpc];
+        tmem_ld8(tlane + (uint32_t)(l * NH + 32 * cq + c), v);
+        f2 h[4];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = gelu(v[j] + bias[l * HID + c0 + j]);
-      put_operand(v, l & 1);
+        for (int j = 0; j < 4; ++j)
+          h[j] = gelu2(z_pair(v[2 * j], v[2 * j + 1], bias + l * HID + c0 + c + 2 * j));
+        put_operand(h, l & 1, c0 + c);
+      }
       publish(l & 1, true);
     }
     if (!ok) break;
@@ -366,7 +403,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     fence_async_smem();
     tc_before_sync();
-    __syncthreads();
+    compute_sync();
     // ---- backward: the pre-activation gradients of layers 2 to 0 ----
 #pragma unroll 1
     for (int l = 2; l >= 0; --l) {
@@ -389,40 +426,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         copy_out(l, a.dZT[l + 1]);
       }
       if (!(ok = sync_mma())) break;
-      float v[32], z[32];
-      tmem_ld32(tlane + dcol + (uint32_t)(32 * cq), v);
-      tmem_ld32(tlane + (uint32_t)(l * NH + 32 * cq), z);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = v[j] * gelu_grad(z[j] + bias[l * HID + c0 + j]);
       // layer 2's gradient goes to buffer 1, layer 1's to 0, layer 0's to 1
       const int buf = (l == 1) ? 0 : 1;
-      put_operand(v, buf);
+#pragma unroll 1
+      for (int c = 0; c < 32; c += kEpc) {
+        float v[kEpc], z[kEpc];
+        tmem_ld8(tlane + dcol + (uint32_t)(32 * cq + c), v);
+        tmem_ld8(tlane + (uint32_t)(l * NH + 32 * cq + c), z);
+        f2 h[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          h[j] = f2_mul(f2_pack(v[2 * j], v[2 * j + 1]),
+                        gelu_grad2(z_pair(z[2 * j], z[2 * j + 1],
+                                          bias + l * HID + c0 + c + 2 * j)));
+        put_operand(h, buf, c0 + c);
+      }
       publish(buf, l > 0);
       if (l == 0) copy_out(buf, a.dZT[0]);
     }
   } while (false);
 
-  if (tid == 0) {
-    if (ok) {
-      // the tensor cores' last arrivals on the slot barriers precede the exit
-      for (int g = kStreamed - NSLOT; g < kStreamed; ++g)
-        mbar_wait(bar_empty + 8 * (g % NSLOT), (g / NSLOT) & 1);
-    } else {
-      // let the tensor-core work and the copies in flight land before the
-      // shared and tensor memory are released
-      mbar_wait(bar_mma, mph ^ 1);
-      for (int g = g_landed; g < g_load; ++g)
-        mbar_wait(bar_full + 8 * (g % NSLOT), (g / NSLOT) & 1);
-      mbar_wait(bar_w3, 0);
-      for (; n_half < n_sent; ++n_half) mbar_wait(bar_half + 8 * (n_half & 1), (n_half >> 1) & 1);
-      atomicExch(a.err, kDevErrNnWait);
-    }
+  if (!ok && tid == 0) {
+    // let the tensor-core work and the peer's copies in flight land before the
+    // shared and tensor memory are released
+    mbar_wait(bar_mma, mph ^ 1);
+    for (; n_half < n_sent; ++n_half) mbar_wait(bar_half + 8 * (n_half & 1), (n_half >> 1) & 1);
+    atomicExch(a.err, kDevErrNnWait);
   }
   tc_before_sync();
   __syncthreads();
   // neither CTA leaves while the other may still send to it
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
+  cluster_sync();
   if (warp == 0) {
     tc_after_sync();
     tmem_free(tmem, 512);
@@ -633,7 +667,7 @@ cudaError_t train_pass(const TrainPassArgs& a, int64_t tiles, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(train_pass_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmem);
   if (e != cudaSuccess) return e;
-  train_pass_kernel<<<(unsigned)(2 * tiles), kThreads, kPassSmem, s>>>(a);
+  train_pass_kernel<<<(unsigned)(2 * tiles), kPassLaunch, kPassSmem, s>>>(a);
   return cudaGetLastError();
 }
 
