@@ -33,7 +33,7 @@ constexpr int kWBand = 32;           // fine points per instrument profile
 constexpr int kWMaxLam = 1024;       // fine grid points
 constexpr int kWChunk = 64;          // fine points per chunk: two per lane
 constexpr int kWMaxChunks = kWMaxLam / kWChunk;
-constexpr int kWWarps = 9;           // pixels in flight per CTA at most
+constexpr int kWWarps = 8;           // pixels in flight per CTA at most
 constexpr int kWBand4 = kWBand + 4;  // a band starting on a multiple of 4, padded to 4
 constexpr int kWBandStride = kWBand4 + 4;  // [lo4, n4, pad, pad, w[36]] per sample
 constexpr int kWWin = 8;             // groups of four points a window holds
@@ -229,7 +229,7 @@ __device__ __forceinline__ void wide_chunk(const Weideman& W, const PixK& P, con
 // loads of four conflict-free rows for its 112 sums and a third of the lanes
 // idle.  Instruction fetch bounds the kernel now (about one stall an issue:
 // warps at different places of 20 KB of loop); rolling the pass' loops to
-// half the code cost more instructions than it saved (43.2 -> 48.0 ms).
+// half the code cost more instructions than it saved (43.3 -> 48.0 ms).
 template <int WD>
 __device__ __forceinline__ void wide_pass_windows(const Weideman& W, const PixK& P,
                                                   const float* xg, const float* win, int g0,
@@ -925,10 +925,11 @@ cudaError_t launch_wide_invert(const InvertArgs& a, int nf, cudaStream_t s) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   nsm = sm_budget(nsm);
-  // one CTA per SM, a pixel a warp: as many warps as the shared memory holds
-  // (9 with 112 samples: 65,536 pixels 41.9 ms, with 8 43.2; halving the
-  // chunk's buffer made room for 12, 43.1), fewer when the map does not fill
-  // them, so that its pixels spread over all SMs
+  // one CTA per SM, a pixel a warp: up to 8 warps (65,536 pixels of 112
+  // samples 43.0 ms; with 9, what the shared memory holds, 43.3; halving the
+  // chunk's buffer made room for 12, 43.1), fewer when a long instrument table
+  // leaves no room or the map does not fill them, so that its pixels spread
+  // over all SMs
   int64_t warps = (a.npix + nsm - 1) / nsm;
   if (warps > kWWarps) warps = kWWarps;
   if (warps < 1) warps = 1;
