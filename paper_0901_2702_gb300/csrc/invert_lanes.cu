@@ -19,10 +19,10 @@
 // Every sum takes its terms in the order, and every element its operations,
 // of invert_kernel with one thread per pixel, so results are the same bits.
 // A 300-pixel map (51 passes) takes 1.15 ms against 4.05 ms of invert_kernel,
-// 4,096 pixels 1.72 against 4.05; about 43 k cycles an iteration, a good
+// 4,096 pixels 1.64 against 4.05; about 43 k cycles an iteration, a good
 // third of them FP64 instructions in a chain.  On maps that fill the chip the
 // FP64 pipe bounds it (300 instructions serve four pixels, 550 serve 32 in
-// the other kernels) and it loses: 1,048,576 pixels 204 ms against 101.
+// the other kernels) and it loses: 1,048,576 pixels 204 ms against 85.
 #include <math.h>
 
 #include "common.cuh"

@@ -79,7 +79,7 @@ constexpr int KX = XT;                            // features padded to two K = 
 constexpr int NY = YN;                            // outputs padded
 // columns an epilogue takes at once, in a rolled loop: a CTA runs each layer's
 // code once or thrice, so that unrolling it costs instruction fetches (a step
-// of 8192 samples takes 75.5 us with 8, 1 more with 16, 4 more with 32)
+// of 8192 samples takes 1 us more of 76 with 16, 4 more with 32)
 constexpr int kEpc = 8;
 constexpr int kPassLaunch = kThreads + 32;  // and a warp that loads the weights
 constexpr int kStreamed = 18;  // weight chunks a tile: W0 1, W1 4, W2 4, W3^T 1, W2^T 4, W1^T 4
@@ -594,13 +594,27 @@ __device__ __forceinline__ void dw_tile(const uint8_t* A, const uint8_t* B, floa
     for (int j = 0; j < 16; j += 4)
       *reinterpret_cast<float4*>(pp + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
   } else {
+    // through the warp's 4 KB of the stages, free by now, so that a store
+    // instruction writes four rows' 128 bytes (16-byte pieces of 32 rows cost
+    // eight times the wavefronts: 16 steps of 8192 samples 1.20 -> 1.08 ms)
+    float4* t = reinterpret_cast<float4*>(sm + warp * 4096);
+    float* prow = P + (size_t)(mt * TMR + 32 * lq) * N + (N == 256 ? cq * 64 : 0);
 #pragma unroll 1
     for (int c = 0; c < (N == 256 ? 64 : N); c += 32) {
       float v[32];
       tmem_ld32(lane_addr + (uint32_t)((N == 256 ? cq * 64 : 0) + c), v);
+      __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 32; j += 4)
-        *reinterpret_cast<float4*>(pp + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      for (int j = 0; j < 8; ++j)
+        t[lane * 8 + (j ^ (lane & 7))] =
+            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = 4 * j + (lane >> 3);
+        *reinterpret_cast<float4*>(prow + (size_t)r * N + c + 4 * (lane & 7)) =
+            t[r * 8 + ((lane & 7) ^ (r & 7))];
+      }
     }
   }
 }
