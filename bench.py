@@ -109,10 +109,9 @@ FLOP_NORMAL_EQ = 24 * 30 + 24 * (9 + 2 * 54)
 TRAFFIC_BYTES_PER_PIXEL = (54_240_512 + 153_698_048) / 262_144
 # The same for the warp-specialised LM kernel (invert_ws_kernel, the shape the
 # autotuner picks): one ncu capture on 1,048,576 pixels of the 1024^2
-# distributions (210.3 MB read + 92.8 MB write; profiles/invert_ws_kernel_1m_px.md):
-# 289 B per pixel, the extra writes over the algorithmic 52 B being the
-# consumers' spilled registers written back.
-TRAFFIC_BYTES_PER_PIXEL_WS = (210_325_504 + 92_827_392) / 1_048_576
+# distributions (207.3 MB read + 40.3 MB write; profiles/invert_ws_kernel_1m_px.md):
+# 236 B per pixel, a part of the outputs staying in L2.
+TRAFFIC_BYTES_PER_PIXEL_WS = (207_335_424 + 40_274_944) / 1_048_576
 LM_KERNEL_FUSED = "invert_kernel<6>"
 LM_KERNEL_WS = "invert_ws_kernel<6> (warp-specialised)"
 
@@ -503,13 +502,12 @@ def run_ours(args, rank, world):
         "gpu_launches": None,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
-                     "traffic": None,
+                     "traffic": (TRAFFIC_BYTES_PER_PIXEL_WS * npix if best_block == 384
+                                 else None),
                      "traffic_note": (
-                         "null: the kernel changed after its last ncu capture (its barrier "
-                         "wait now returns the warp's vote; no memory access changed); that "
-                         f"capture of 1,048,576 pixels read+wrote {TRAFFIC_BYTES_PER_PIXEL_WS:.0f} "
-                         "B/px against the algorithmic 244 (reads 201 vs 192, writes 89 vs 52), "
-                         f"{TRAFFIC_BYTES_PER_PIXEL_WS * npix:.3g} B for this launch"
+                         f"{TRAFFIC_BYTES_PER_PIXEL_WS:.0f} B/px read+written by an ncu capture "
+                         "of 1,048,576 pixels (198 + 38; algorithmic 192 + 52, a part of the "
+                         "outputs staying in L2), times this launch's pixels"
                          if best_block == 384 else
                          "null: the kernel changed after its last ncu capture (63-point table, "
                          "normal-equation changes); that capture of 262,144 pixels at 79 points "

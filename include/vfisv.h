@@ -272,8 +272,8 @@ void vfisv_graph_destroy(vfisv_graph* g);
  * workload asks for pixels per CTA and threads per pixel to be tuned): time
  * an inversion of the given sample (arguments as vfisv_invert, no
  * covariance) with 64, 128 and 256 threads per CTA and 1, 2 and 4 threads
- * per pixel, and with the warp-specialised kernel (384 threads per CTA, one
- * pixel per thread of its two consumer warpgroups, one CTA per SM), keep the
+ * per pixel, and with the warp-specialised kernel (384 threads per CTA, up to
+ * 384 pixels in flight, one CTA per SM), keep the
  * fastest shape for this handle's later inversions and return it in
  * best_block (threads per CTA) and best_tpp (threads per pixel, may be
  * NULL); ms_out (may be NULL) receives the ten times: ms_out[3 * i + j] for
@@ -282,8 +282,8 @@ void vfisv_graph_destroy(vfisv_graph* g);
  * points: a pass has tpp times as many threads, so small maps (fewer pixels
  * than resident slots) finish sooner, while the solve and the normal
  * equations are repeated on every lane of the pixel.  The warp-specialised
- * kernel runs the wavelength pass in one warpgroup and the chi2, normal
- * equations and FP64 solve in the other two, handing the filtered rows over
+ * kernel is a pipeline of three warpgroups -- the wavelength pass; chi2 and
+ * the normal equations; the FP64 solve -- handing the filtered rows over
  * through tensor memory; it takes the default configuration (restarts, a
  * free filling factor and fast_solve run the 128 x 1 kernel instead).
  * Results do not
@@ -327,7 +327,7 @@ int vfisv_set_pipeline_chunks(vfisv_handle* h, int32_t chunks);
  * device error is a bounded wait (about a second) that gave up: the filter
  * table's copy into shared memory, a network operand copy or tensor-core
  * completion, a filtered-row buffer of the one-warpgroup LM kernel, or a
- * producer/consumer hand-off of the warp-specialised LM kernel.  The kernel
+ * hand-off between the stages of the warp-specialised LM kernel.  The kernel
  * then stops and returns, so the context stays usable, but the outputs of
  * the calls since the last check are not valid.  The error words are
  * cleared. */
