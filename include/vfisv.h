@@ -298,9 +298,10 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
  * block in {64, 128, 256} threads per CTA with tpp in {1, 2, 4} threads per
  * pixel, or block = 384 with tpp = 1 for the warp-specialised kernel.  Until a
  * shape is set (here or by vfisv_autotune) the library chooses by the size of
- * the map: a kernel with eight lanes per pixel for maps of up to about 15,000
- * pixels, the warp-specialised one above; results are the same
- * bits as with 128 x 1.  VFISV_E_ARG for any other value. */
+ * the map: a kernel with eight lanes per pixel for maps of up to about 12,900
+ * pixels, above them the warp-specialised one, or 128 x 1 on long
+ * wavelength grids where that is faster; results are the same bits.
+ * VFISV_E_ARG for any other value. */
 int vfisv_set_launch_shape(vfisv_handle* h, int32_t block, int32_t tpp);
 
 /* Persistent launches of this handle (the LM, wide, covariance and network

@@ -1016,6 +1016,22 @@ static cudaError_t invert_slots_t(int nlam, int64_t npix, int restarts, int64_t*
   }
 }
 
+// Without a set shape: whether the warp-specialised kernel (else 128 x 1) takes
+// a map of npix pixels on nsm SMs.  128 x 1 has up to two CTAs, 256 pixels an
+// SM, in flight; the other 384, but one producer warp a sub-partition makes
+// their passes, the longer part on a long grid: there 128 x 1 is faster up to
+// one CTA an SM, and again above two until the pipeline is full.  Measured
+// (ms, 128 x 1 / warp-specialised): up to 128 pixels an SM 3.81 / 3.71 on 149
+// points, 3.88 / 3.98 on 175, 5.10 / 5.33 on 297; up to 256 the latter always
+// (30,000 pixels 8.87 / 7.72 on 297, 14.9 / 14.2 on 600); 40,000 pixels 9.16 /
+// 9.05 on 225, 9.72 / 10.17 on 260, 13.2 / 16.0 on 450; 50,000 12.7 / 11.4 on
+// 297, 16.2 / 16.3 on 450; 130,000 27.8 / 26.1 on 350, 40.3 / 42.2 on 600.
+static bool ws_by_size(int nlam, int64_t npix, int64_t nsm) {
+  if (npix <= 128 * nsm) return nlam <= 160;
+  if (npix <= 256 * nsm || nlam <= 230) return true;
+  return (nlam <= 320 && npix > 300 * nsm) || (nlam <= 400 && npix > 640 * nsm);
+}
+
 cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_solve,
                          int alpha_free, int64_t* nslots, int* grid, int* block, int* tpp,
                          size_t* smem) {
@@ -1028,12 +1044,12 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
   }
   const bool plain = !restarts && !fast_solve;
   if (*block == 0) {
-    // no shape set: by the pixels an SM gets.  Several lanes a pixel up to
-    // 100 (15,200 pixels on 152 SMs), the warp-specialised kernel above.
-    // Measured (ms; lanes / 128 x 1 / warp-specialised): 300 pixels 1.16 /
-    // 3.82 / 3.73, 4,096 1.64 / 4.06 / -, 12,288 3.26 / 3.85 / 3.77, 17,000
-    // - / 3.86 / 3.77, 19,000 5.38 / 3.86 / 3.77, 40,000 8.96 / 8.06 / 6.64,
-    // 1,048,576 204 / 138 / 85.
+    // no shape set: by the pixels an SM gets.  Several lanes a pixel up to 85
+    // (12,920 pixels on 152 SMs), above that by ws_by_size().  Measured (ms;
+    // lanes / 128 x 1 / warp-specialised): 300 pixels 1.16 / 3.82 / 3.73, 4,096
+    // 1.64 / 4.06 / -, 12,000 3.22 / 3.82 / 3.71 (75 points 2.70 / 4.01 / 2.90,
+    // 297 points 4.48 / 5.11 / 5.32), 15,000 3.91 / 3.82 / 3.72 (75 points 3.32
+    // / 4.10 / 2.90), 40,000 8.96 / 8.06 / 6.64, 1,048,576 204 / 138 / 85.
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -1043,11 +1059,12 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
     if (plain) {
       // (a long filter table leaves room for few one-warp CTAs: those maps
       // must then fit twice over)
-      if (npix <= 100 * (int64_t)nsm &&
+      if (npix <= 85 * (int64_t)nsm &&
           invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
           npix <= 2 * *nslots)
         *block = kInvLanesBlock;
-      else if (invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
+      else if (ws_by_size(nlam, npix, nsm) &&
+               invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
         *block = kInvWsBlock;
       cudaGetLastError();
     }

@@ -133,3 +133,17 @@ def test_same_bits_in_a_replayed_graph(pair):
             for k in out:
                 assert torch.equal(out[k], ref[k]), k
     g.close()
+
+
+@pytest.mark.parametrize("nlam,per_sm", [(160, 85), (160, 128), (161, 128), (230, 256),
+                                         (231, 256), (320, 300), (321, 300), (400, 640),
+                                         (401, 640)])
+@pytest.mark.parametrize("extra", [0, 1])
+def test_same_bits_at_the_lines_of_the_rule(pair, nlam, per_sm, extra):
+    # pixels an SM and wavelength points where the kernel chosen changes
+    v, torch, a, b = pair
+    n = 8 * per_sm + extra
+    x = np.linspace(-740.0, 740.0, nlam)
+    p, obs, w, tf, tx = _map(v, a, torch, n, nlam + n, T_=W.hmi_filters(x), X_=x)
+    v.vfisv_set_sm_limit(a, 8)
+    _equal(v, torch, a, b, lambda h: v.vfisv_invert(h, obs, w, tf, tx, LINE))
