@@ -935,8 +935,11 @@ cudaError_t launch_wide_invert(const InvertArgs& a, int nf, cudaStream_t s) {
   if (warps < 1) warps = 1;
   while (warps > 1 && wide_smem(nf, a.nlam, true, (int)warps) > (size_t)most) --warps;
   const size_t smem = wide_smem(nf, a.nlam, true, (int)warps);
+  // the limit belongs to the kernel, not to the call, and the warps, so the
+  // bytes, go by the map: with the call's own bytes as the limit, a thread with
+  // a small map lowered it between another's setting and launch, which then failed
   cudaError_t e = cudaFuncSetAttribute(wide_invert_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
   int64_t g = (a.npix + warps - 1) / warps;
   if (g > nsm) g = nsm;
