@@ -230,8 +230,9 @@ cudaError_t launch_synth(const SynthArgs& a, int nf, cudaStream_t s);
 // Persistent LM kernel: launch shape for `npix` pixels with *block threads
 // per CTA (64, 128 or 256; anything else selects 128) and *tpp threads per
 // pixel (1, 2 or 4; anything else selects 1), both written back as used
-// (restarts and a free filling factor take 128 x 1), and the number of
-// resident pixel slots (the scratch it needs): grid x block / tpp.
+// (restarts and a free filling factor take 128 x 1), and the number of pixel
+// slots the workspace has to hold scratch for: the resident ones (grid x block
+// / tpp), or those of 128 x 1 where the kernel needs none.
 cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_solve,
                          int alpha_free, int64_t* nslots, int* grid, int* block, int* tpp,
                          size_t* smem);

@@ -1072,8 +1072,15 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
   if (*block == kInvLanesBlock || *block == kInvWsBlock) {
     if (plain) {
       *tpp = 1;
-      return *block == kInvWsBlock ? invert_ws_slots(nlam, npix, nslots, grid, smem)
-                                   : invert_lanes_slots(nlam, npix, nslots, grid, smem);
+      // Both keep their normal equations in shared memory, but the workspace
+      // has room for 128 x 1 all the same: it then goes by the map's size
+      // alone, and a handle that has run a map runs, or captures, any smaller
+      // one without growing it, whichever of the kernels that one takes.
+      cudaError_t e = slots_for<kInvThreadsDefault, false, false>(nlam, npix, nslots, grid, smem);
+      if (e != cudaSuccess) return e;
+      int64_t own = 0;
+      return *block == kInvWsBlock ? invert_ws_slots(nlam, npix, &own, grid, smem)
+                                   : invert_lanes_slots(nlam, npix, &own, grid, smem);
     }
     *block = kInvThreadsDefault;  // not compiled for this configuration
   }
