@@ -299,8 +299,9 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
  * pixel, or block = 384 with tpp = 1 for the warp-specialised kernel.  Until a
  * shape is set (here or by vfisv_autotune) the library chooses by the size of
  * the map: a kernel with eight lanes per pixel for maps of up to about 12,900
- * pixels, above them the warp-specialised one, or 128 x 1 on long
- * wavelength grids where that is faster; results are the same bits.
+ * pixels, above them the warp-specialised one, or 128 x 1 where the filters
+ * keep so many grid points that this is faster (a choice made on the device);
+ * results are the same bits.
  * VFISV_E_ARG for any other value. */
 int vfisv_set_launch_shape(vfisv_handle* h, int32_t block, int32_t tpp);
 

@@ -475,10 +475,10 @@ int invert_device(vfisv_handle* h, const DevInvert& d, int nfilt, int nlam,
   int64_t nslots = 0;
   int grid = 0, block = h->lm_block, tpp = h->lm_tpp;
   size_t smem = 0;
+  LmBeyond beyond;
   const bool alpha_free = (cfg->free_mask >> 9) & 1u;
   if (invert_slots(nfilt, nlam, npix, cfg->restarts, cfg->fast_solve, alpha_free, &nslots, &grid,
-                   &block, &tpp, &smem) !=
-      cudaSuccess) {
+                   &block, &tpp, &smem, &beyond) != cudaSuccess) {
     cudaGetLastError();
     return VFISV_E_CUDA;
   }
@@ -543,7 +543,14 @@ int invert_device(vfisv_handle* h, const DevInvert& d, int nfilt, int nlam,
   a.rs_state = cfg->restarts ? ws + L.rs : nullptr;
   a.pix_list = d.pix_list;
   a.counters = h->counters;
+  if (beyond.rows < nlam) a.rows_max = beyond.rows;
   if (launch_invert(a, nfilt, grid, block, tpp, smem, s) != cudaSuccess) return VFISV_E_CUDA;
+  if (beyond.rows < nlam) {
+    a.rows_min = beyond.rows + 1;
+    a.rows_max = INT_MAX;
+    if (launch_invert(a, nfilt, beyond.grid, kInvThreadsDefault, 1, beyond.smem, s) != cudaSuccess)
+      return VFISV_E_CUDA;
+  }
   // with a pixel list the listed pixels lie anywhere in [0, npix): the
   // covariance kernel sweeps the whole map (it skips rows by status)
   if (d.cov && !d.park_cov &&

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include "me_device.cuh"
@@ -166,6 +167,9 @@ struct InvertArgs {
   // optional list of the pixels to invert: queue position q inverts pixel
   // pix_list[q] (q < *npix_dev); the others are not touched
   const int64_t* pix_list = nullptr;
+  // the launch does nothing unless the filter table keeps rows_min .. rows_max
+  // rows (LmBeyond)
+  int rows_min = 0, rows_max = INT_MAX;
   // optional work counters, added to by every CTA when it exits:
   // [0] fused passes (each trial model, plus the starting model),
   // [1] accepted trials (each followed by a J^T W J build), [2] pixels
@@ -175,6 +179,13 @@ struct InvertArgs {
 
 constexpr int kScratchPerSlot = 45 + 9;  // packed J^T W J and J^T W r
 constexpr int kScratchPerSlotAlpha = 55 + 10;  // the same with the filling factor free
+
+// The same answer on every thread of the grid, before anything is loaded.
+__device__ __forceinline__ bool rows_wanted(const InvertArgs& A, int nf) {
+  if (A.rows_min == 0 && A.rows_max == INT_MAX) return true;
+  const int r = table_rows(A.table, nf, A.nlam);
+  return r >= A.rows_min && r <= A.rows_max;
+}
 
 // Map of a pixel in a batch (binary search over the prefix offsets).
 __device__ __forceinline__ int map_of(const int64_t* off, int nmaps, int64_t pix) {
@@ -227,15 +238,25 @@ constexpr int kRestartAtConvergence = 1, kRestartA = 2, kRestartB = 4;
 cudaError_t launch_pack_table(const float* filters, int nf, const float* wl, int nlam,
                               float* table, cudaStream_t s);
 cudaError_t launch_synth(const SynthArgs& a, int nf, cudaStream_t s);
+constexpr int kInvThreadsDefault = 128;
 // Persistent LM kernel: launch shape for `npix` pixels with *block threads
 // per CTA (64, 128 or 256; anything else selects 128) and *tpp threads per
 // pixel (1, 2 or 4; anything else selects 1), both written back as used
 // (restarts and a free filling factor take 128 x 1), and the number of pixel
 // slots the workspace has to hold scratch for: the resident ones (grid x block
 // / tpp), or those of 128 x 1 where the kernel needs none.
+// *block = 0 lets the size of the map choose (`beyond` not null).  Where that
+// depends on the rows the filter table keeps, which only the device knows, the
+// kernel chosen takes tables of up to beyond->rows of them and a second launch,
+// of 128 x 1 with beyond's grid, the others: one of the two returns at once.
+struct LmBeyond {
+  int rows = INT_MAX;  // no second launch unless below the table's points
+  int grid = 0;
+  size_t smem = 0;
+};
 cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_solve,
                          int alpha_free, int64_t* nslots, int* grid, int* block, int* tpp,
-                         size_t* smem);
+                         size_t* smem, LmBeyond* beyond = nullptr);
 cudaError_t launch_restart_perturb(const float* in, int64_t n, int64_t pix0, int k,
                                    uint32_t free_mask, uint64_t seed, float* out, cudaStream_t s);
 // Upload the Weideman coefficients to the LM kernel's constant bank on the
@@ -247,6 +268,7 @@ cudaError_t invert_set_constants(const Weideman& W);
 // restarts, filling factor held).
 constexpr int kInvWsBlock = 384;
 cudaError_t invert_ws_set_constants(const Weideman& W);
+bool invert_ws_three(int nlam);  // three batches a sub-partition fit beside the table
 cudaError_t invert_ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem);
 cudaError_t launch_invert_ws(const InvertArgs& a, int grid, size_t smem, cudaStream_t s);
 // The kernel for maps too small to fill the chip one pixel a thread

@@ -17,7 +17,6 @@
 
 namespace vfisv {
 
-constexpr int kInvThreadsDefault = 128;  // pixel slots per CTA unless autotuned
 
 // The same factorisation and solve in double-float arithmetic (the fast
 // path of the damped step; FP64 is kept for the rare singular fallback).
@@ -380,6 +379,7 @@ __global__ void __launch_bounds__(BS, 1) invert_kernel(InvertArgs A) {
   constexpr int NP = AF ? 10 : kNP;        // parameters in the solve
   constexpr int NPK = NP * (NP + 1) / 2;   // packed J^T W J
   extern __shared__ __align__(16) float smem[];
+  if (!rows_wanted(A, NF)) return;
   const int S = table_stride(NF);
   const int tabf = table_floats(NF, A.nlam);
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -1016,25 +1016,36 @@ static cudaError_t invert_slots_t(int nlam, int64_t npix, int restarts, int64_t*
   }
 }
 
-// Without a set shape: whether the warp-specialised kernel (else 128 x 1) takes
-// a map of npix pixels on nsm SMs.  128 x 1 has up to two CTAs, 256 pixels an
-// SM, in flight; the other 384, but one producer warp a sub-partition makes
-// their passes, the longer part on a long grid: there 128 x 1 is faster up to
-// one CTA an SM, and again above two until the pipeline is full.  Measured
-// (ms, 128 x 1 / warp-specialised): up to 128 pixels an SM 3.81 / 3.71 on 149
-// points, 3.88 / 3.98 on 175, 5.10 / 5.33 on 297; up to 256 the latter always
-// (30,000 pixels 8.87 / 7.72 on 297, 14.9 / 14.2 on 600); 40,000 pixels 9.16 /
-// 9.05 on 225, 9.72 / 10.17 on 260, 13.2 / 16.0 on 450; 50,000 12.7 / 11.4 on
-// 297, 16.2 / 16.3 on 450; 130,000 27.8 / 26.1 on 350, 40.3 / 42.2 on 600.
-static bool ws_by_size(int nlam, int64_t npix, int64_t nsm) {
-  if (npix <= 128 * nsm) return nlam <= 160;
-  if (npix <= 256 * nsm || nlam <= 230) return true;
-  return (nlam <= 320 && npix > 300 * nsm) || (nlam <= 400 && npix > 640 * nsm);
+// Without a set shape: the filter-table rows up to which the warp-specialised
+// kernel (else 128 x 1) takes a map of npix pixels on nsm SMs; 0: none.  128 x 1
+// has up to two CTAs, 256 pixels an SM, in flight; the other 384, but one
+// producer warp a sub-partition makes their passes, the longer part when the
+// table keeps many rows: how much a second wave costs either of them goes by
+// the pixels an SM.  The rows, not the grid's points: the same filters keep 63
+// of 149 points and all of a grid that is cut to their support.  Measured, time
+// of the pipeline over 128 x 1's, by pixels an SM and kept rows:
+//      86 - 128: 63 rows 0.97, 70 1.02, 100 1.04, 230 1.06
+//           129: 190 0.97, 230 1.00, 300 1.03         256: 230 0.91, 300 0.99
+//           257: 80 0.95, 90 1.01, 149 1.21, 230 1.30
+//           300: 125 0.98, 140 1.00      384: 230 0.92      500: 160 0.99, 180 1.02
+//     560 - 700: 110 0.97, 125 1.00           1,200: 140 0.95, 160 0.99, 180 1.03
+//         6,900: 63 0.63, 125 0.87, 160 0.94
+// A table that leaves room for two batches only: 200 pixels an SM 0.97 (200 rows
+// of 3,000 points), 256 0.79 to 0.90; 129 1.18 (64 of 3,000), and beyond 256 128 x 1
+// has one CTA an SM too, so it is left to that.
+static int ws_rows(int nlam, int64_t npix, int64_t nsm) {
+  if (!invert_ws_three(nlam)) return (npix >= 200 * nsm && npix <= 256 * nsm) ? 200 : 0;
+  if (npix <= 128 * nsm) return 66;
+  if (npix <= 256 * nsm) return 230;
+  if (npix <= 300 * nsm) return 85;
+  if (npix <= 550 * nsm) return 130;
+  if (npix <= 750 * nsm) return 118;
+  return 150;
 }
 
 cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_solve,
                          int alpha_free, int64_t* nslots, int* grid, int* block, int* tpp,
-                         size_t* smem) {
+                         size_t* smem, LmBeyond* beyond) {
   if (nf != 6) return cudaErrorInvalidValue;
   if (alpha_free) {  // compiled for the default slot count, FP64 solve, no restarts
     if (restarts || fast_solve) return cudaErrorInvalidValue;
@@ -1045,28 +1056,34 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
   const bool plain = !restarts && !fast_solve;
   if (*block == 0) {
     // no shape set: by the pixels an SM gets.  Several lanes a pixel up to 85
-    // (12,920 pixels on 152 SMs), above that by ws_by_size().  Measured (ms;
+    // (12,920 pixels on 152 SMs), above that by ws_rows().  Measured (ms;
     // lanes / 128 x 1 / warp-specialised): 300 pixels 1.16 / 3.82 / 3.73, 4,096
     // 1.64 / 4.06 / -, 12,000 3.22 / 3.82 / 3.71 (75 points 2.70 / 4.01 / 2.90,
     // 297 points 4.48 / 5.11 / 5.32), 15,000 3.91 / 3.82 / 3.72 (75 points 3.32
     // / 4.10 / 2.90), 40,000 8.96 / 8.06 / 6.64, 1,048,576 204 / 138 / 85.
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    nsm = sm_budget(nsm);
     *block = kInvThreadsDefault;
     *tpp = 1;
-    if (plain) {
+    if (plain && beyond) {
+      int dev = 0, nsm = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      nsm = sm_budget(nsm);
+      auto fits = [](cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess;
+      };
       // (a long filter table leaves room for few one-warp CTAs: those maps
       // must then fit twice over)
-      if (npix <= 85 * (int64_t)nsm &&
-          invert_lanes_slots(nlam, npix, nslots, grid, smem) == cudaSuccess &&
-          npix <= 2 * *nslots)
+      if (npix <= 85 * (int64_t)nsm && fits(invert_lanes_slots(nlam, npix, nslots, grid, smem)) &&
+          npix <= 2 * *nslots) {
         *block = kInvLanesBlock;
-      else if (ws_by_size(nlam, npix, nsm) &&
-               invert_ws_slots(nlam, npix, nslots, grid, smem) == cudaSuccess)
-        *block = kInvWsBlock;
-      cudaGetLastError();
+      } else {
+        const int rows = ws_rows(nlam, npix, nsm);
+        if (rows > 0 && fits(invert_ws_slots(nlam, npix, nslots, grid, smem))) {
+          *block = kInvWsBlock;
+          beyond->rows = rows;
+        }
+      }
     }
   }
   if (*block == kInvLanesBlock || *block == kInvWsBlock) {
@@ -1076,7 +1093,9 @@ cudaError_t invert_slots(int nf, int nlam, int64_t npix, int restarts, int fast_
       // has room for 128 x 1 all the same: it then goes by the map's size
       // alone, and a handle that has run a map runs, or captures, any smaller
       // one without growing it, whichever of the kernels that one takes.
-      cudaError_t e = slots_for<kInvThreadsDefault, false, false>(nlam, npix, nslots, grid, smem);
+      LmBeyond other;
+      LmBeyond& o = beyond ? *beyond : other;
+      cudaError_t e = slots_for<kInvThreadsDefault, false, false>(nlam, npix, nslots, &o.grid, &o.smem);
       if (e != cudaSuccess) return e;
       int64_t own = 0;
       return *block == kInvWsBlock ? invert_ws_slots(nlam, npix, &own, grid, smem)

@@ -593,6 +593,7 @@ __global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A,
   static_assert(kProdRegs % 8 == 0 && kAccRegs<NB> % 8 == 0 && kSolveRegs<NB> % 8 == 0,
                 "setmaxnreg counts");
   extern __shared__ __align__(16) float smem[];
+  if (!rows_wanted(A, NF)) return;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int tabf = table_floats(NF, A.nlam);
   const WsSmem<NB> L(tabf);
@@ -674,9 +675,9 @@ cudaError_t invert_ws_set_constants(const Weideman& W) {
 }
 
 // Three batches a sub-partition where the slots' state fits beside the filter
-// table, else two (tables of more than about 3,000 points).
+// table, else two (tables of more than 1,584 points).
 constexpr size_t kWsSmemMax = 227 * 1024;
-static bool ws_three(int nlam) {
+bool invert_ws_three(int nlam) {
   return WsSmem<kWsBatches>(table_floats(6, nlam)).total <= kWsSmemMax;
 }
 
@@ -715,7 +716,7 @@ static cudaError_t ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, 
 }
 
 cudaError_t invert_ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem) {
-  return ws_three(nlam) ? ws_slots<kWsBatches>(nlam, npix, nslots, grid, smem)
+  return invert_ws_three(nlam) ? ws_slots<kWsBatches>(nlam, npix, nslots, grid, smem)
                         : ws_slots<2>(nlam, npix, nslots, grid, smem);
 }
 
@@ -724,7 +725,7 @@ cudaError_t launch_invert_ws(const InvertArgs& a, int grid, size_t smem, cudaStr
   // that its pixels spread over all SMs
   const int64_t per = (int64_t)grid * kWsGroups * 32;
   const int64_t want = (a.npix + per - 1) / per;
-  const int most = ws_three(a.nlam) ? kWsBatches : 2;
+  const int most = invert_ws_three(a.nlam) ? kWsBatches : 2;
   const int nb = want < 1 ? 1 : (want > most ? most : (int)want);
   if (most == kWsBatches)
     invert_ws_kernel<6, kWsBatches><<<grid, kWsThreadsN, smem, s>>>(a, nb);

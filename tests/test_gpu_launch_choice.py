@@ -47,3 +47,45 @@ def test_a_smaller_map_needs_no_larger_workspace(vf, nlam, big, small):  # noqa:
     v.vfisv_check(h)
     g.close()
     h.close()
+
+
+def _ms(torch, call, reps=6):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for i in range(reps):
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        if i:
+            best = min(best, a.elapsed_time(b))
+    return best
+
+
+# points of the grid, half its span (mA; the filters end at 310: nothing beyond
+# is kept), pixels an SM, most that the call may take of 128 x 1's time
+@pytest.mark.parametrize("nlam,half,per_sm,most", [
+    (80, 310.0, 110, 1.1), (149, 310.0, 257, 1.1), (230, 310.0, 258, 1.1), (190, 310.0, 640, 1.1),
+    (600, 310.0, 256, 1.1), (2500, 310.0, 150, 1.1), (3000, 14500.0, 129, 1.1),
+    # few points kept: the warp-specialised kernel's gain has to stay
+    (149, 740.0, 200, 0.9), (600, 2900.0, 257, 0.95), (1700, 8300.0, 256, 0.85)])
+def test_the_choice_goes_by_the_points_kept(vf, nlam, half, per_sm, most):  # noqa: F811
+    """A pass costs the grid points that the filter table keeps, not those of
+    the grid: on grids cut to the filters' support as on wide ones, a call
+    without a set shape is no slower than 128 x 1, and the same bits (margin:
+    10 %; choosing by the grid's points lost up to 57 % here)."""
+    v, _, torch = vf
+    a, b = v.vfisv_create(0), v.vfisv_create(0)
+    v.vfisv_set_launch_shape(b, 128, 1)
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    obs, w, tf, tx = _map(v, a, torch, n, np.linspace(-half, half, nlam))
+    out = [v.vfisv_invert(h, obs, w, tf, tx, LINE, want_cov=False) for h in (a, b)]
+    for k in out[0]:
+        assert out[0][k] is None or torch.equal(out[0][k], out[1][k]), k
+    ms = [_ms(torch, lambda: v.vfisv_invert(h, obs, w, tf, tx, LINE, want_cov=False, out=o))
+          for h, o in zip((a, b), out)]
+    print(f"{nlam} points to {half} mA, {per_sm} pixels an SM: {ms[0]:.2f} / {ms[1]:.2f} ms")
+    assert ms[0] <= most * ms[1], ms
+    for h in (a, b):
+        v.vfisv_check(h)
+        h.close()
