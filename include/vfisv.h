@@ -272,12 +272,16 @@ void vfisv_graph_destroy(vfisv_graph* g);
  * workload asks for pixels per CTA and threads per pixel to be tuned): time
  * an inversion of the given sample (arguments as vfisv_invert, no
  * covariance) with 64, 128 and 256 threads per CTA and 1, 2 and 4 threads
- * per pixel, and with the warp-specialised kernel (384 threads per CTA, up to
- * 384 pixels in flight, one CTA per SM), keep the
+ * per pixel, with the warp-specialised kernel (384 threads per CTA, up to
+ * 384 pixels in flight, one CTA per SM), and, where that is yet another
+ * kernel, with the library's choice by the map's size
+ * (vfisv_set_launch_shape); keep the
  * fastest shape for this handle's later inversions and return it in
  * best_block (threads per CTA) and best_tpp (threads per pixel, may be
- * NULL); ms_out (may be NULL) receives the ten times: ms_out[3 * i + j] for
+ * NULL), 0 and 1 when the choice by size was the fastest; ms_out (may be NULL)
+ * receives the ten shapes' times: ms_out[3 * i + j] for
  * tpp = {1, 2, 4}[i], block = {64, 128, 256}[j], then ms_out[9] for 384 x 1.
+ * When a run fails its error is returned and the handle keeps the shape it had.
  * With tpp threads per pixel the lanes of a pixel split its wavelength
  * points: a pass has tpp times as many threads, so small maps (fewer pixels
  * than resident slots) finish sooner, while the solve and the normal
@@ -296,7 +300,8 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
 
 /* Set the launch shape of the handle's filter-position LM kernel directly:
  * block in {64, 128, 256} threads per CTA with tpp in {1, 2, 4} threads per
- * pixel, or block = 384 with tpp = 1 for the warp-specialised kernel.  Until a
+ * pixel, block = 384 with tpp = 1 for the warp-specialised kernel, or block = 0
+ * with tpp = 1 to go back to no shape.  Until a
  * shape is set (here or by vfisv_autotune) the library chooses by the size of
  * the map: a kernel with eight lanes per pixel for maps of up to about 12,900
  * pixels, above them the warp-specialised one, or 128 x 1 where the filters

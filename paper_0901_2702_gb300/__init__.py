@@ -486,7 +486,8 @@ def vfisv_graph_destroy(g: Graph) -> None:
 def vfisv_autotune(h: Handle, obs, weights, filters, wl_mA, line, config=None, stream=None):
     """Pick the LM kernel's launch shape on a sample; returns (threads per CTA,
     threads per pixel, [ms x 10]: threads-per-pixel-major over 64/128/256 x
-    1/2/4, then the warp-specialised 384 x 1)."""
+    1/2/4, then the warp-specialised 384 x 1).  (0, 1): no shape, the choice by
+    the map's size is faster than all of them."""
     npix = int(obs.shape[0])
     nfilt, nlam = int(filters.shape[0]), int(filters.shape[1])
     per_pixel = 1 if (len(weights.shape) >= 2 and int(weights.shape[0]) == npix) else 0
@@ -504,7 +505,8 @@ def vfisv_autotune(h: Handle, obs, weights, filters, wl_mA, line, config=None, s
 
 def vfisv_set_launch_shape(h: Handle, block: int, tpp: int = 1) -> None:
     """Threads per CTA (64, 128, 256) and per pixel (1, 2, 4) of the LM kernel,
-    or 384 x 1: the warp-specialised kernel."""
+    384 x 1: the warp-specialised kernel, or 0 x 1: the library's choice by the
+    map's size (a new handle's)."""
     _check(load().vfisv_set_launch_shape(h.ptr, int(block), int(tpp)), "vfisv_set_launch_shape")
 
 

@@ -766,18 +766,35 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
   char* mw = (char*)h->mixws;
   // threads per CTA x threads per pixel, threads-per-pixel-major, then the
   // warp-specialised kernel (kInvWsBlock threads, one pixel per consumer
-  // thread)
+  // thread), then the choice by the map's size (0 x 1)
   const int cand_b[3] = {64, 128, 256}, cand_t[3] = {1, 2, 4};
+  constexpr int kShapes = 10;  // those that ms_out reports
   auto shape = [&](int c, int* b, int* t) {
-    *b = (c < 9) ? cand_b[c % 3] : kInvWsBlock;
+    *b = (c < 9) ? cand_b[c % 3] : (c < kShapes ? kInvWsBlock : 0);
     *t = (c < 9) ? cand_t[c / 3] : 1;
   };
+  const int old_b = h->lm_block, old_t = h->lm_tpp;
   float best = 0.0f;
-  int best_b = 128, best_t = 1;
+  int best_b = old_b, best_t = old_t;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  for (int c = 0; c < 10; ++c) {
+  for (int c = 0; c <= kShapes; ++c) {
+    if (c == kShapes) {
+      // the choice by size is a candidate where it takes a kernel that has no
+      // shape of its own (eight lanes per pixel; the arguments are checked by now)
+      int64_t ns = 0;
+      int g = 0, b = 0, t = 1;
+      size_t sm = 0;
+      LmBeyond beyond;
+      if (nfilt != 6 || invert_slots(nfilt, nlam, npix, cfg->restarts, cfg->fast_solve,
+                                     (cfg->free_mask >> 9) & 1u, &ns, &g, &b, &t, &sm,
+                                     &beyond) != cudaSuccess) {
+        cudaGetLastError();
+        break;
+      }
+      if (b != kInvLanesBlock) break;
+    }
     shape(c, &h->lm_block, &h->lm_tpp);
     float ms = 0.0f;
     for (int rep = 0; rep < 2; ++rep) {  // the first run warms up
@@ -791,7 +808,7 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
       cudaEventElapsedTime(&ms, e0, e1);
     }
     if (rc) break;
-    if (ms_out) ms_out[c] = ms;
+    if (ms_out && c < kShapes) ms_out[c] = ms;
     if (c == 0 || ms < best) {
       best = ms;
       shape(c, &best_b, &best_t);
@@ -799,16 +816,17 @@ int vfisv_autotune(vfisv_handle* h, const float* obs, const float* weights,
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  h->lm_block = best_b;
-  h->lm_tpp = best_t;
-  *best_block = best_b;
-  if (best_tpp) *best_tpp = best_t;
+  // a run that failed leaves the handle as it was
+  h->lm_block = rc ? old_b : best_b;
+  h->lm_tpp = rc ? old_t : best_t;
+  *best_block = h->lm_block;
+  if (best_tpp) *best_tpp = h->lm_tpp;
   return rc;
 }
 
 int vfisv_set_launch_shape(vfisv_handle* h, int32_t block, int32_t tpp) {
   const bool plain = (block == 64 || block == 128 || block == 256) && (tpp == 1 || tpp == 2 || tpp == 4);
-  if (!h || !(plain || (block == kInvWsBlock && tpp == 1))) return VFISV_E_ARG;
+  if (!h || !(plain || ((block == kInvWsBlock || block == 0) && tpp == 1))) return VFISV_E_ARG;
   h->lm_block = block;
   h->lm_tpp = tpp;
   return VFISV_OK;
