@@ -762,7 +762,8 @@ __global__ void __launch_bounds__(BS, 1) invert_kernel(InvertArgs A) {
 // J^T W J parked in the pixel's output row ----
 
 // The eigen-decomposition fallback of one pixel by kNP lanes: jacobi_pinv() and
-// the scaling around it with every element's operations in the same order,
+// the scaling around it with every element's operations in the same order and
+// the same roundings (both spell them out),
 // row k of the matrix and of the eigenvectors on lane k, the rotations'
 // angles on all of them.  A lane alone spends two thirds of a rotation's
 // FP64 time on the 3 kNP pairs of elements that these lanes update together, so a few
@@ -812,52 +813,38 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
     double off = 0.0, dia = 0.0;
     if (run)
       for (int i = 0; i < N; ++i) {
-        dia += B.a[i][i] * B.a[i][i];
-        for (int j = i + 1; j < N; ++j) off += B.a[i][j] * B.a[i][j];
+        dia = fma(B.a[i][i], B.a[i][i], dia);
+        for (int j = i + 1; j < N; ++j) off = fma(B.a[i][j], B.a[i][j], off);
       }
-    if (!(off > 1e-26 * dia)) run = false;
+    if (!(off > __dmul_rn(1e-26, dia))) run = false;
     if (!__any_sync(0xffffffffu, run)) break;
     for (int p = 0; p < N - 1; ++p)
       for (int q = p + 1; q < N; ++q) {
         const double apq = B.a[p][q], app = B.a[p][p], aqq = B.a[q][q];
         const bool act = run && apq != 0.0;
-        double c = 1.0, sn = 0.0;
-        if (act) {
-          const double th = (aqq - app) / (2.0 * apq);
-          const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-          c = 1.0 / sqrt(t * t + 1.0);
-          sn = t * c;
-        }
+        Rotation r{1.0, 0.0};
+        if (act) r = jacobi_rotation(apq, app, aqq);
         __syncwarp();  // the pivots are read before they change
         if (act) {
-          const double akp = B.a[k][p], akq = B.a[k][q];
-          const double vkp = B.v[k][p], vkq = B.v[k][q];
-          B.a[k][p] = c * akp - sn * akq;
-          B.a[k][q] = sn * akp + c * akq;
-          B.v[k][p] = c * vkp - sn * vkq;
-          B.v[k][q] = sn * vkp + c * vkq;
+          r.apply(B.a[k][p], B.a[k][q]);
+          r.apply(B.v[k][p], B.v[k][q]);
         }
         __syncwarp();
-        if (act) {
-          const double apk = B.a[p][k], aqk = B.a[q][k];
-          B.a[p][k] = c * apk - sn * aqk;
-          B.a[q][k] = sn * apk + c * aqk;
-        }
+        if (act) r.apply(B.a[p][k], B.a[q][k]);
         __syncwarp();
       }
   }
   if (live) {
     double lmax = 0.0;
     for (int i = 0; i < N; ++i) lmax = fmax(lmax, fabs(B.a[i][i]));
-    const double l = fabs(B.a[k][k]);
-    B.li[k] = (l > 1e-12 * lmax && l > 0.0) ? 1.0 / B.a[k][k] : 0.0;
+    B.li[k] = jacobi_inverse(B.a[k][k], lmax);
   }
   __syncwarp();
   if (live) {
     // row k of the lower triangle, unscaled, and its mirror image
     for (int j = 0; j <= k; ++j) {
       double s = 0.0;
-      for (int e = 0; e < N; ++e) s += B.v[k][e] * B.li[e] * B.v[j][e];
+      for (int e = 0; e < N; ++e) s = fma(__dmul_rn(B.v[k][e], B.li[e]), B.v[j][e], s);
       const float q = ((held >> k) & 1u) || ((held >> j) & 1u) ? 0.0f
                                                                : (float)(B.sc[k] * B.sc[j] * s);
       row[k * 10 + j] = q;
@@ -891,10 +878,8 @@ __global__ void __launch_bounds__(kCovThreads) covariance_kernel(float* cov,
                                                                  const int64_t* npix_dev,
                                                                  uint32_t free_mask, int ppr) {
   __shared__ int32_t queue[kCovQueue];  // pixel = queue / ppr * stride + base + queue % ppr
-  // with the filling factor free every singular pixel takes the one-lane path:
-  // there the groups' results differ from it in the last bits (the compiler
-  // fuses other products of the rotations), and a row's bits must not depend
-  // on the map it came in
+  // with the filling factor free (10 parameters) every singular pixel takes the
+  // one-lane path
   constexpr bool kCoop = NPAR == kNP;
   __shared__ CoopPixel coop[kCoop ? kCoopMax : 1];
   __shared__ int qn;

@@ -41,11 +41,39 @@ __device__ __forceinline__ double eps_update(double e, bool success) {
   return fmax(n, 1e-9);  // floor: the scaled damped matrix keeps eigenvalues >= 1e-9
 }
 
+// A Jacobi rotation, with every rounding written out unless it is PLAIN (there
+// the compiler chooses which product of a sum it fuses).
+struct Rotation {
+  double c, s;
+  template <bool PLAIN = false>
+  __device__ __forceinline__ void apply(double& p, double& q) const {
+    const double x = p, y = q;
+    p = PLAIN ? c * x - s * y : fma(c, x, -__dmul_rn(s, y));
+    q = PLAIN ? s * x + c * y : fma(s, x, __dmul_rn(c, y));
+  }
+};
+__device__ __forceinline__ Rotation jacobi_rotation(double apq, double app, double aqq) {
+  const double th = (aqq - app) / __dmul_rn(2.0, apq);
+  const double t = (th >= 0.0 ? 1.0 : -1.0) / __dadd_rn(fabs(th), sqrt(fma(th, th, 1.0)));
+  const double c = 1.0 / sqrt(fma(t, t, 1.0));
+  return {c, __dmul_rn(t, c)};
+}
+// The reciprocal of an eigenvalue, zero below 1e-12 of the largest.
+__device__ __forceinline__ double jacobi_inverse(double e, double lmax) {
+  const double l = fabs(e);
+  return (l > __dmul_rn(1e-12, lmax) && l > 0.0) ? 1.0 / e : 0.0;
+}
+
 // Symmetric eigen-decomposition by cyclic Jacobi rotations, FP64; the
 // fallback when the Cholesky pivots show a (numerically) singular matrix.
 // Solves M y = b with eigenvalues below 1e-12 * max zeroed (truncated SVD
 // of a symmetric matrix), or, with b == nullptr, writes the truncated
 // pseudo-inverse into Minv.
+// Every rounding is written out (fma, __dmul_rn): covariance_coop() takes the
+// same steps spread over lanes, a pixel's path there depends on the queue, and
+// its bits must not depend on which products a compiler chooses to fuse.  The
+// rotations with 10 parameters, which have this path alone, keep the plain
+// expressions that their results come from.
 template <int N = kNP>
 static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, const double* b,
                                          double* y, double* Minv) {
@@ -58,58 +86,42 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
   for (int sweep = 0; sweep < 30; ++sweep) {
     double off = 0.0, dia = 0.0;
     for (int i = 0; i < N; ++i) {
-      dia += a[i][i] * a[i][i];
-      for (int j = i + 1; j < N; ++j) off += a[i][j] * a[i][j];
+      dia = fma(a[i][i], a[i][i], dia);
+      for (int j = i + 1; j < N; ++j) off = fma(a[i][j], a[i][j], off);
     }
-    if (!(off > 1e-26 * dia)) break;  // off-diagonal below ~3e-13 of the diagonal
+    if (!(off > __dmul_rn(1e-26, dia))) break;  // off-diagonal below ~3e-13 of the diagonal
     for (int p = 0; p < N - 1; ++p)
       for (int q = p + 1; q < N; ++q) {
         const double apq = a[p][q];
         if (apq == 0.0) continue;
-        const double th = (a[q][q] - a[p][p]) / (2.0 * apq);
-        const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-        const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-        for (int k = 0; k < N; ++k) {
-          const double akp = a[k][p], akq = a[k][q];
-          a[k][p] = c * akp - s * akq;
-          a[k][q] = s * akp + c * akq;
-        }
-        for (int k = 0; k < N; ++k) {
-          const double apk = a[p][k], aqk = a[q][k];
-          a[p][k] = c * apk - s * aqk;
-          a[q][k] = s * apk + c * aqk;
-        }
-        for (int k = 0; k < N; ++k) {
-          const double vkp = v[k][p], vkq = v[k][q];
-          v[k][p] = c * vkp - s * vkq;
-          v[k][q] = s * vkp + c * vkq;
-        }
+        const Rotation r = jacobi_rotation(apq, a[p][p], a[q][q]);
+        constexpr bool P = N != kNP;
+        for (int k = 0; k < N; ++k) r.apply<P>(a[k][p], a[k][q]);
+        for (int k = 0; k < N; ++k) r.apply<P>(a[p][k], a[q][k]);
+        for (int k = 0; k < N; ++k) r.apply<P>(v[k][p], v[k][q]);
       }
   }
   double lmax = 0.0;
   for (int i = 0; i < N; ++i) lmax = fmax(lmax, fabs(a[i][i]));
   double linv[N];
-  for (int i = 0; i < N; ++i) {
-    const double l = fabs(a[i][i]);
-    linv[i] = (l > 1e-12 * lmax && l > 0.0) ? 1.0 / a[i][i] : 0.0;
-  }
+  for (int i = 0; i < N; ++i) linv[i] = jacobi_inverse(a[i][i], lmax);
   if (b) {
     double t[N];
     for (int i = 0; i < N; ++i) {
       double s = 0.0;
-      for (int k = 0; k < N; ++k) s += v[k][i] * b[k];
-      t[i] = s * linv[i];
+      for (int k = 0; k < N; ++k) s = fma(v[k][i], b[k], s);
+      t[i] = __dmul_rn(s, linv[i]);
     }
     for (int k = 0; k < N; ++k) {
       double s = 0.0;
-      for (int i = 0; i < N; ++i) s += v[k][i] * t[i];
+      for (int i = 0; i < N; ++i) s = fma(v[k][i], t[i], s);
       y[k] = s;
     }
   } else {
     for (int i = 0; i < N; ++i)
       for (int j = 0; j <= i; ++j) {
         double s = 0.0;
-        for (int k = 0; k < N; ++k) s += v[i][k] * linv[k] * v[j][k];
+        for (int k = 0; k < N; ++k) s = fma(__dmul_rn(v[i][k], linv[k]), v[j][k], s);
         Minv[tri(i, j)] = s;
       }
   }
@@ -290,7 +302,7 @@ __device__ __forceinline__ void damped_step_fp64_body(const float* scr, int64_t 
     bv[i] = held[i] ? 0.0 : (double)scr[(int64_t)((N * (N + 1) / 2) + i) * ns] * sc[i];
   jacobi_pinv<N>(L, bv, y, nullptr);
 #pragma unroll
-  for (int i = 0; i < N; ++i) delta[i] = held[i] ? 0.0 : sc[i] * y[i];
+  for (int i = 0; i < N; ++i) delta[i] = held[i] ? 0.0 : __dmul_rn(sc[i], y[i]);
 }
 
 // The same step kept out of line (the LM kernel that calls it from the
