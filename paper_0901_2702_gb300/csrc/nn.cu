@@ -38,10 +38,10 @@ __device__ __forceinline__ void put_bf16(uint8_t* base, size_t off, float v) {
   *reinterpret_cast<bf16*>(base + off) = __float2bfloat16(v);
 }
 
-__constant__ LayerDim kLayers[4] = {{IN, HID, K0P, HID, OFF_W0, OFF_B0},
-                                    {HID, HID, HID, HID, OFF_W1, OFF_B1},
-                                    {HID, HID, HID, HID, OFF_W2, OFF_B2},
-                                    {HID, OUT, HID, N3P, OFF_W3, OFF_B3}};
+__constant__ LayerDim kLayers[4] = {{IN, HID, OFF_W0, OFF_B0},
+                                    {HID, HID, OFF_W1, OFF_B1},
+                                    {HID, HID, OFF_W2, OFF_B2},
+                                    {HID, OUT, OFF_W3, OFF_B3}};
 
 // End of a step: sums the split-K partials (fixed order: deterministic) and,
 // ADAM, applies the update with bias correction (m = b1 m + (1-b1) g,

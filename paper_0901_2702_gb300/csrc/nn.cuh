@@ -12,8 +12,6 @@ namespace vfisv {
 namespace nn {
 
 constexpr int IN = VFISV_NN_NIN, HID = VFISV_NN_NHID, OUT = VFISV_NN_NOUT;
-constexpr int K0P = 64;      // input width padded for the tensor-core tiles
-constexpr int N3P = 64;      // output width padded likewise
 constexpr int kSplits = 32;  // most split-K CTAs per tile of the weight-gradient products
 
 constexpr size_t OFF_W0 = 0;
@@ -33,13 +31,9 @@ constexpr size_t NTRAIN = OFF_INM;  // weights and biases (trained)
 static_assert(NBLOB == VFISV_NN_NBLOB, "blob layout");
 
 struct LayerDim {
-  int K, N, Kp, Np;
+  int K, N;
   size_t offW, offB;
 };
-constexpr LayerDim kLayersHost[4] = {{IN, HID, K0P, HID, OFF_W0, OFF_B0},
-                                     {HID, HID, HID, HID, OFF_W1, OFF_B1},
-                                     {HID, HID, HID, HID, OFF_W2, OFF_B2},
-                                     {HID, OUT, HID, N3P, OFF_W3, OFF_B3}};
 
 // Affine permutation of sample indices: sample(m) = (mult (offset + m) + add) mod n.
 struct Perm {

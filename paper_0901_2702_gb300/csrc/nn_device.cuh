@@ -12,18 +12,9 @@
 namespace vfisv {
 namespace nn {
 
-// GELU(x) = x Phi(x) and its derivative Phi(x) + x phi(x).
-__device__ __forceinline__ float gelu(float x) {
-  return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));
-}
-__device__ __forceinline__ float gelu_grad(float x) {
-  const float cdf = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
-  const float pdf = 0.39894228040143268f * expf(-0.5f * x * x);
-  return fmaf(x, pdf, cdf);
-}
-
-// The same, two at a time: what surrounds the error function and the
-// exponential in packed instructions (the same roundings).
+// GELU(x) = x Phi(x) = 0.5 x (1 + erf(x / sqrt(2))) and its derivative Phi(x) +
+// x phi(x), two at a time: what surrounds the error function and the
+// exponential in packed instructions (the scalar ones' roundings).
 __device__ __forceinline__ f2 gelu2(f2 x) {
   const f2 t = f2_mul(x, f2_dup(0.70710678118654752f));
   const f2 e = f2_pack(erff(f2_lo(t)), erff(f2_hi(t)));
