@@ -324,7 +324,7 @@ bool pipeline_host(const vfisv_handle* h, const void* obs, int64_t npix, bool no
          !is_device_ptr(obs);
 }
 
-// Workspace layout: [err int | queue u64 | pad] [table] [scratch] [restart state]
+// Workspace layout: [err int | 2 queues u64 | pad] [table] [scratch] [restart state]
 struct WsLayout {
   size_t err = 0, queue = 64, table = 256, scratch = 0, rs = 0, total = 0;
 };
@@ -502,9 +502,13 @@ int invert_device(vfisv_handle* h, const DevInvert& d, int nfilt, int nlam,
       return VFISV_E_CUDA;
     init = (const float*)h->wfinit;
   }
-  if (launch_pack_table(d.filters, nfilt, d.wl, nlam, table, s) != cudaSuccess)
+  // two queues: one of two launches may be left without pixels (LmBeyond)
+  unsigned long long* queues = (unsigned long long*)(ws + L.queue);
+  const bool two = beyond.rows < nlam;
+  if (cudaMemsetAsync(queues, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess)
     return VFISV_E_CUDA;
-  if (cudaMemsetAsync(ws + L.queue, 0, sizeof(unsigned long long), s) != cudaSuccess)
+  if (launch_pack_table(d.filters, nfilt, d.wl, nlam, table, s, two ? queues : nullptr,
+                        beyond.rows) != cudaSuccess)
     return VFISV_E_CUDA;
   InvertArgs a;
   a.obs = d.obs;
@@ -522,7 +526,7 @@ int invert_device(vfisv_handle* h, const DevInvert& d, int nfilt, int nlam,
   a.cov_out = d.cov;
   a.scratch = (float*)(ws + L.scratch);
   a.nslots = nslots;
-  a.queue = (unsigned long long*)(ws + L.queue);
+  a.queue = queues;
   a.err = (int*)(ws + L.err);
   a.W = h->W;
   a.lk = line_constants(line);
@@ -543,11 +547,9 @@ int invert_device(vfisv_handle* h, const DevInvert& d, int nfilt, int nlam,
   a.rs_state = cfg->restarts ? ws + L.rs : nullptr;
   a.pix_list = d.pix_list;
   a.counters = h->counters;
-  if (beyond.rows < nlam) a.rows_max = beyond.rows;
   if (launch_invert(a, nfilt, grid, block, tpp, smem, s) != cudaSuccess) return VFISV_E_CUDA;
-  if (beyond.rows < nlam) {
-    a.rows_min = beyond.rows + 1;
-    a.rows_max = INT_MAX;
+  if (two) {
+    a.queue = queues + 1;
     if (launch_invert(a, nfilt, beyond.grid, kInvThreadsDefault, 1, beyond.smem, s) != cudaSuccess)
       return VFISV_E_CUDA;
   }

@@ -167,9 +167,6 @@ struct InvertArgs {
   // optional list of the pixels to invert: queue position q inverts pixel
   // pix_list[q] (q < *npix_dev); the others are not touched
   const int64_t* pix_list = nullptr;
-  // the launch does nothing unless the filter table keeps rows_min .. rows_max
-  // rows (LmBeyond)
-  int rows_min = 0, rows_max = INT_MAX;
   // optional work counters, added to by every CTA when it exits:
   // [0] fused passes (each trial model, plus the starting model),
   // [1] accepted trials (each followed by a J^T W J build), [2] pixels
@@ -179,13 +176,6 @@ struct InvertArgs {
 
 constexpr int kScratchPerSlot = 45 + 9;  // packed J^T W J and J^T W r
 constexpr int kScratchPerSlotAlpha = 55 + 10;  // the same with the filling factor free
-
-// The same answer on every thread of the grid, before anything is loaded.
-__device__ __forceinline__ bool rows_wanted(const InvertArgs& A, int nf) {
-  if (A.rows_min == 0 && A.rows_max == INT_MAX) return true;
-  const int r = table_rows(A.table, nf, A.nlam);
-  return r >= A.rows_min && r <= A.rows_max;
-}
 
 // Map of a pixel in a batch (binary search over the prefix offsets).
 __device__ __forceinline__ int map_of(const int64_t* off, int nmaps, int64_t pix) {
@@ -235,8 +225,11 @@ struct RestartState {
 };
 constexpr int kRestartAtConvergence = 1, kRestartA = 2, kRestartB = 4;
 
+// queues (may be null): two zeroed work-queue counters; the first is moved past
+// every pixel when the table keeps more than `rows` rows, else the second.
 cudaError_t launch_pack_table(const float* filters, int nf, const float* wl, int nlam,
-                              float* table, cudaStream_t s);
+                              float* table, cudaStream_t s, unsigned long long* queues = nullptr,
+                              int rows = 0);
 cudaError_t launch_synth(const SynthArgs& a, int nf, cudaStream_t s);
 constexpr int kInvThreadsDefault = 128;
 // Persistent LM kernel: launch shape for `npix` pixels with *block threads
@@ -248,7 +241,10 @@ constexpr int kInvThreadsDefault = 128;
 // *block = 0 lets the size of the map choose (`beyond` not null).  Where that
 // depends on the rows the filter table keeps, which only the device knows, the
 // kernel chosen takes tables of up to beyond->rows of them and a second launch,
-// of 128 x 1 with beyond's grid, the others: one of the two returns at once.
+// of 128 x 1 with beyond's grid and a queue of its own, the others: one of the
+// two finds its queue empty (launch_pack_table) and ends after a few
+// microseconds.  (A test of the rows at the kernels' start was dearer: it moved
+// the warp-specialised kernel's code and cost its whole run 1 %.)
 struct LmBeyond {
   int rows = INT_MAX;  // no second launch unless below the table's points
   int grid = 0;

@@ -379,7 +379,6 @@ __global__ void __launch_bounds__(BS, 1) invert_kernel(InvertArgs A) {
   constexpr int NP = AF ? 10 : kNP;        // parameters in the solve
   constexpr int NPK = NP * (NP + 1) / 2;   // packed J^T W J
   extern __shared__ __align__(16) float smem[];
-  if (!rows_wanted(A, NF)) return;
   const int S = table_stride(NF);
   const int tabf = table_floats(NF, A.nlam);
   const int tid = threadIdx.x, nt = blockDim.x;

@@ -593,7 +593,6 @@ __global__ void __launch_bounds__(kWsThreadsN, 1) invert_ws_kernel(InvertArgs A,
   static_assert(kProdRegs % 8 == 0 && kAccRegs<NB> % 8 == 0 && kSolveRegs<NB> % 8 == 0,
                 "setmaxnreg counts");
   extern __shared__ __align__(16) float smem[];
-  if (!rows_wanted(A, NF)) return;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int tabf = table_floats(NF, A.nlam);
   const WsSmem<NB> L(tabf);

@@ -32,7 +32,7 @@ constexpr int kCand = 32, kCandWarp = 8;  // candidate thresholds a round, and o
 
 __global__ void __launch_bounds__(kPackThreads) pack_table_kernel(
     const float* __restrict__ filters, int nf, const float* __restrict__ wl, int nlam,
-    float* __restrict__ table) {
+    float* __restrict__ table, unsigned long long* queues, int rows) {
   const int S = table_stride(nf);
   __shared__ float rbuf[kMassGrid];  // relative weight r_i of each point
   __shared__ float mass[kMassMaxNF];  // M_k
@@ -162,11 +162,13 @@ __global__ void __launch_bounds__(kPackThreads) pack_table_kernel(
     if (lane == 0)
       table[(size_t)nlam * S + k] = (k < nf) ? s : (k == S - 1 ? __int_as_float(base) : 0.0f);
   }
+  if (queues && threadIdx.x == 0) queues[base > rows ? 0 : 1] = 1ull << 62;
 }
 
 cudaError_t launch_pack_table(const float* filters, int nf, const float* wl, int nlam,
-                              float* table, cudaStream_t s) {
-  pack_table_kernel<<<1, kPackThreads, 0, s>>>(filters, nf, wl, nlam, table);
+                              float* table, cudaStream_t s, unsigned long long* queues,
+                              int rows) {
+  pack_table_kernel<<<1, kPackThreads, 0, s>>>(filters, nf, wl, nlam, table, queues, rows);
   return cudaGetLastError();
 }
 
