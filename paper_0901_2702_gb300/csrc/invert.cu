@@ -815,7 +815,7 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
         dia = fma(B.a[i][i], B.a[i][i], dia);
         for (int j = i + 1; j < N; ++j) off = fma(B.a[i][j], B.a[i][j], off);
       }
-    if (!(off > __dmul_rn(1e-26, dia))) run = false;
+    if (!(off > 1e-26 * dia)) run = false;
     if (!__any_sync(0xffffffffu, run)) break;
     for (int p = 0; p < N - 1; ++p)
       for (int q = p + 1; q < N; ++q) {
@@ -825,11 +825,22 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
         if (act) r = jacobi_rotation(apq, app, aqq);
         __syncwarp();  // the pivots are read before they change
         if (act) {
-          r.apply(B.a[k][p], B.a[k][q]);
-          r.apply(B.v[k][p], B.v[k][q]);
+          double akp = B.a[k][p], akq = B.a[k][q];
+          double vkp = B.v[k][p], vkq = B.v[k][q];
+          r.apply(akp, akq);
+          r.apply(vkp, vkq);
+          B.a[k][p] = akp;
+          B.a[k][q] = akq;
+          B.v[k][p] = vkp;
+          B.v[k][q] = vkq;
         }
         __syncwarp();
-        if (act) r.apply(B.a[p][k], B.a[q][k]);
+        if (act) {
+          double apk = B.a[p][k], aqk = B.a[q][k];
+          r.apply(apk, aqk);
+          B.a[p][k] = apk;
+          B.a[q][k] = aqk;
+        }
         __syncwarp();
       }
   }
@@ -843,7 +854,7 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
     // row k of the lower triangle, unscaled, and its mirror image
     for (int j = 0; j <= k; ++j) {
       double s = 0.0;
-      for (int e = 0; e < N; ++e) s = fma(__dmul_rn(B.v[k][e], B.li[e]), B.v[j][e], s);
+      for (int e = 0; e < N; ++e) s = fma(B.v[k][e] * B.li[e], B.v[j][e], s);
       const float q = ((held >> k) & 1u) || ((held >> j) & 1u) ? 0.0f
                                                                : (float)(B.sc[k] * B.sc[j] * s);
       row[k * 10 + j] = q;

@@ -41,27 +41,28 @@ __device__ __forceinline__ double eps_update(double e, bool success) {
   return fmax(n, 1e-9);  // floor: the scaled damped matrix keeps eigenvalues >= 1e-9
 }
 
-// A Jacobi rotation, with every rounding written out unless it is PLAIN (there
-// the compiler chooses which product of a sum it fuses).
+// A Jacobi rotation.  Every sum of products is an fma(), so that no rounding is
+// left to the compiler, unless it is PLAIN (there it chooses which product of a
+// sum it fuses).
 struct Rotation {
   double c, s;
   template <bool PLAIN = false>
   __device__ __forceinline__ void apply(double& p, double& q) const {
     const double x = p, y = q;
-    p = PLAIN ? c * x - s * y : fma(c, x, -__dmul_rn(s, y));
-    q = PLAIN ? s * x + c * y : fma(s, x, __dmul_rn(c, y));
+    p = PLAIN ? c * x - s * y : fma(c, x, -(s * y));
+    q = PLAIN ? s * x + c * y : fma(s, x, c * y);
   }
 };
 __device__ __forceinline__ Rotation jacobi_rotation(double apq, double app, double aqq) {
-  const double th = (aqq - app) / __dmul_rn(2.0, apq);
-  const double t = (th >= 0.0 ? 1.0 : -1.0) / __dadd_rn(fabs(th), sqrt(fma(th, th, 1.0)));
+  const double th = (aqq - app) / (2.0 * apq);
+  const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(fma(th, th, 1.0)));
   const double c = 1.0 / sqrt(fma(t, t, 1.0));
-  return {c, __dmul_rn(t, c)};
+  return {c, t * c};
 }
 // The reciprocal of an eigenvalue, zero below 1e-12 of the largest.
 __device__ __forceinline__ double jacobi_inverse(double e, double lmax) {
   const double l = fabs(e);
-  return (l > __dmul_rn(1e-12, lmax) && l > 0.0) ? 1.0 / e : 0.0;
+  return (l > 1e-12 * lmax && l > 0.0) ? 1.0 / e : 0.0;
 }
 
 // Symmetric eigen-decomposition by cyclic Jacobi rotations, FP64; the
@@ -69,8 +70,8 @@ __device__ __forceinline__ double jacobi_inverse(double e, double lmax) {
 // Solves M y = b with eigenvalues below 1e-12 * max zeroed (truncated SVD
 // of a symmetric matrix), or, with b == nullptr, writes the truncated
 // pseudo-inverse into Minv.
-// Every rounding is written out (fma, __dmul_rn): covariance_coop() takes the
-// same steps spread over lanes, a pixel's path there depends on the queue, and
+// Every sum of products is written as fma(): covariance_coop() takes the same
+// steps spread over lanes, a pixel's path there depends on the queue, and
 // its bits must not depend on which products a compiler chooses to fuse.  The
 // rotations with 10 parameters, which have this path alone, keep the plain
 // expressions that their results come from.
@@ -89,7 +90,7 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
       dia = fma(a[i][i], a[i][i], dia);
       for (int j = i + 1; j < N; ++j) off = fma(a[i][j], a[i][j], off);
     }
-    if (!(off > __dmul_rn(1e-26, dia))) break;  // off-diagonal below ~3e-13 of the diagonal
+    if (!(off > 1e-26 * dia)) break;  // off-diagonal below ~3e-13 of the diagonal
     for (int p = 0; p < N - 1; ++p)
       for (int q = p + 1; q < N; ++q) {
         const double apq = a[p][q];
@@ -110,7 +111,7 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
     for (int i = 0; i < N; ++i) {
       double s = 0.0;
       for (int k = 0; k < N; ++k) s = fma(v[k][i], b[k], s);
-      t[i] = __dmul_rn(s, linv[i]);
+      t[i] = s * linv[i];
     }
     for (int k = 0; k < N; ++k) {
       double s = 0.0;
@@ -121,7 +122,7 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
     for (int i = 0; i < N; ++i)
       for (int j = 0; j <= i; ++j) {
         double s = 0.0;
-        for (int k = 0; k < N; ++k) s = fma(__dmul_rn(v[i][k], linv[k]), v[j][k], s);
+        for (int k = 0; k < N; ++k) s = fma(v[i][k] * linv[k], v[j][k], s);
         Minv[tri(i, j)] = s;
       }
   }
