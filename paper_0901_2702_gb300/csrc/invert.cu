@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(BS, 1) invert_kernel(InvertArgs A) {
 
 // The eigen-decomposition fallback of one pixel by kNP lanes: jacobi_pinv() and
 // the scaling around it with every element's operations in the same order and
-// the same roundings (both spell them out),
+// the same products fused (Rotation),
 // row k of the matrix and of the eigenvectors on lane k, the rotations'
 // angles on all of them.  A lane alone spends two thirds of a rotation's
 // FP64 time on the 3 kNP pairs of elements that these lanes update together, so a few
@@ -812,8 +812,8 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
     double off = 0.0, dia = 0.0;
     if (run)
       for (int i = 0; i < N; ++i) {
-        dia = fma(B.a[i][i], B.a[i][i], dia);
-        for (int j = i + 1; j < N; ++j) off = fma(B.a[i][j], B.a[i][j], off);
+        dia += B.a[i][i] * B.a[i][i];
+        for (int j = i + 1; j < N; ++j) off += B.a[i][j] * B.a[i][j];
       }
     if (!(off > 1e-26 * dia)) run = false;
     if (!__any_sync(0xffffffffu, run)) break;
@@ -854,7 +854,7 @@ __device__ __noinline__ void covariance_coop(CoopPixel* bufs, float* row, uint32
     // row k of the lower triangle, unscaled, and its mirror image
     for (int j = 0; j <= k; ++j) {
       double s = 0.0;
-      for (int e = 0; e < N; ++e) s = fma(B.v[k][e] * B.li[e], B.v[j][e], s);
+      for (int e = 0; e < N; ++e) s += B.v[k][e] * B.li[e] * B.v[j][e];
       const float q = ((held >> k) & 1u) || ((held >> j) & 1u) ? 0.0f
                                                                : (float)(B.sc[k] * B.sc[j] * s);
       row[k * 10 + j] = q;

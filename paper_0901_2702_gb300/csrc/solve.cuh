@@ -41,9 +41,8 @@ __device__ __forceinline__ double eps_update(double e, bool success) {
   return fmax(n, 1e-9);  // floor: the scaled damped matrix keeps eigenvalues >= 1e-9
 }
 
-// A Jacobi rotation.  Every sum of products is an fma(), so that no rounding is
-// left to the compiler, unless it is PLAIN (there it chooses which product of a
-// sum it fuses).
+// A Jacobi rotation.  Which of its sums' two products is fused is written out,
+// unless it is PLAIN (there the compiler chooses).
 struct Rotation {
   double c, s;
   template <bool PLAIN = false>
@@ -70,11 +69,11 @@ __device__ __forceinline__ double jacobi_inverse(double e, double lmax) {
 // Solves M y = b with eigenvalues below 1e-12 * max zeroed (truncated SVD
 // of a symmetric matrix), or, with b == nullptr, writes the truncated
 // pseudo-inverse into Minv.
-// Every sum of products is written as fma(): covariance_coop() takes the same
-// steps spread over lanes, a pixel's path there depends on the queue, and
-// its bits must not depend on which products a compiler chooses to fuse.  The
-// rotations with 10 parameters, which have this path alone, keep the plain
-// expressions that their results come from.
+// covariance_coop() takes the same steps spread over lanes and a pixel's path
+// there depends on the queue, so its bits must not depend on which products a
+// compiler chooses to fuse: the rotations spell that out (the other sums have
+// one product a term, the same choice in both).  With 10 parameters there is
+// this path alone, and the plain expressions that its results come from.
 template <int N = kNP>
 static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, const double* b,
                                          double* y, double* Minv) {
@@ -87,8 +86,8 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
   for (int sweep = 0; sweep < 30; ++sweep) {
     double off = 0.0, dia = 0.0;
     for (int i = 0; i < N; ++i) {
-      dia = fma(a[i][i], a[i][i], dia);
-      for (int j = i + 1; j < N; ++j) off = fma(a[i][j], a[i][j], off);
+      dia += a[i][i] * a[i][i];
+      for (int j = i + 1; j < N; ++j) off += a[i][j] * a[i][j];
     }
     if (!(off > 1e-26 * dia)) break;  // off-diagonal below ~3e-13 of the diagonal
     for (int p = 0; p < N - 1; ++p)
@@ -110,19 +109,19 @@ static __device__ __noinline__ void jacobi_pinv(const double* Mp /*packed*/, con
     double t[N];
     for (int i = 0; i < N; ++i) {
       double s = 0.0;
-      for (int k = 0; k < N; ++k) s = fma(v[k][i], b[k], s);
+      for (int k = 0; k < N; ++k) s += v[k][i] * b[k];
       t[i] = s * linv[i];
     }
     for (int k = 0; k < N; ++k) {
       double s = 0.0;
-      for (int i = 0; i < N; ++i) s = fma(v[k][i], t[i], s);
+      for (int i = 0; i < N; ++i) s += v[k][i] * t[i];
       y[k] = s;
     }
   } else {
     for (int i = 0; i < N; ++i)
       for (int j = 0; j <= i; ++j) {
         double s = 0.0;
-        for (int k = 0; k < N; ++k) s = fma(v[i][k] * linv[k], v[j][k], s);
+        for (int k = 0; k < N; ++k) s += v[i][k] * linv[k] * v[j][k];
         Minv[tri(i, j)] = s;
       }
   }
