@@ -242,7 +242,7 @@ constexpr int kInvThreadsDefault = 128;
 // depends on the rows the filter table keeps, which only the device knows, the
 // kernel chosen takes tables of up to beyond->rows of them and a second launch,
 // of 128 x 1 with beyond's grid and a queue of its own, the others: one of the
-// two finds its queue empty (launch_pack_table) and ends after a few
+// two finds its queue empty (launch_pack_table) and ends after about ten
 // microseconds.  (A test of the rows at the kernels' start was dearer: it moved
 // the warp-specialised kernel's code and cost its whole run 1 %.)
 struct LmBeyond {

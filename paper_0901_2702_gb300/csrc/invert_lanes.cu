@@ -18,8 +18,8 @@
 //             instead of 550, each holding the pipe 64 cycles).
 // Every sum takes its terms in the order, and every element its operations,
 // of invert_kernel with one thread per pixel, so results are the same bits.
-// A 300-pixel map (51 passes) takes 1.15 ms against 4.05 ms of invert_kernel,
-// 4,096 pixels 1.64 against 4.05; about 43 k cycles an iteration, a good
+// A 300-pixel map (51 passes) takes 1.16 ms against 3.82 ms of invert_kernel,
+// 4,096 pixels 1.64 against 4.06; about 43 k cycles an iteration, a good
 // third of them FP64 instructions in a chain.  On maps that fill the chip the
 // FP64 pipe bounds it (300 instructions serve four pixels, 550 serve 32 in
 // the other kernels) and it loses: 1,048,576 pixels 204 ms against 85.

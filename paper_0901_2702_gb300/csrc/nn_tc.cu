@@ -79,7 +79,8 @@ constexpr int KX = XT;                            // features padded to two K = 
 constexpr int NY = YN;                            // outputs padded
 // columns an epilogue takes at once, in a rolled loop: a CTA runs each layer's
 // code once or thrice, so that unrolling it costs instruction fetches (a step
-// of 8192 samples takes 1 us more of 76 with 16, 4 more with 32)
+// of 8192 samples, 76 us when this was measured and 68 now, took 1 us more with
+// 16, 4 more with 32)
 constexpr int kEpc = 8;
 constexpr int kPassLaunch = kThreads + 32;  // and a warp that loads the weights
 constexpr int kStreamed = 18;  // weight chunks a tile: W0 1, W1 4, W2 4, W3^T 1, W2^T 4, W1^T 4
