@@ -69,6 +69,11 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* win = table + wide_common(nf, nlam);
   float* bands = win + wide_win_floats(nlam);
+  // a window reaches past its sample's band, with zero weights, and the points
+  // there must not come out as NaN: no windows on a grid with NaN or far-off
+  // values (padding; up to 1e12 mA the squares stay in range)
+  bool near = true;
+  for (int i = threadIdx.x; i < nlam; i += blockDim.x) near = near && fabsf(wl[i]) < 1e12f;
   for (int k = warp; k < nf; k += blockDim.x >> 5) {
     const float* row = filters + (size_t)k * nlam;
     // first and last non-zero point; tau in a fixed order (lane-strided
@@ -106,7 +111,7 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
     for (int t = lane; t < kWBand4; t += 32)
       b[4 + t] = (t < n4 && lo4 + t < nlam) ? row[lo4 + t] : 0.0f;
   }
-  __syncthreads();
+  const bool ordinary = __syncthreads_and(near);
   // regular bands: sample k's within the window of groups k + start, k +
   // start + width - 1, for every sample
   if (warp == 0) {
@@ -119,7 +124,7 @@ __global__ void wide_pack_kernel(const float* __restrict__ filters, int nf,
     for (int o = 16; o > 0; o >>= 1) g1 = max(g1, __shfl_xor_sync(0xffffffffu, g1, o));
     if (lane == 0) {
       // (every sample's window meets the grid: kernels for 7 and 8 groups)
-      const bool ok = g1 > g0 && g1 - g0 <= kWWin &&
+      const bool ok = ordinary && g1 > g0 && g1 - g0 <= kWWin &&
                       g0 > (g1 - g0 < kWWin ? -(kWWin - 1) : -kWWin) &&
                       g0 + nf <= wide_groups(nlam);
       start = g0;
