@@ -16,6 +16,17 @@ namespace vfisv {
 extern thread_local int t_sm_limit;
 inline int sm_budget(int nsm) { return (t_sm_limit > 0 && t_sm_limit < nsm) ? t_sm_limit : nsm; }
 
+// The dynamic shared memory that kernels whose bytes go by the call (table, map)
+// are allowed: the device's limit.  It is an attribute of the kernel, so with
+// the call's own bytes there a thread whose call needs fewer lowered it between
+// another's setting and launch, which then failed.
+inline int shared_memory_limit() {
+  int dev = 0, most = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return most;
+}
+
 // Device error codes written to the handle's error word.
 enum : int {
   kDevErrNone = 0,

@@ -963,7 +963,8 @@ static cudaError_t slots_for(int nlam, int64_t npix, int64_t* nslots, int* grid,
   constexpr int NPS = BS / TPP;  // pixel slots per CTA
   const size_t sm =
       invert_smem_bytes(table_floats(6, nlam), kRows * 4 * 6 + (AF ? kNmRows * 6 : 0), BS, NPS);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       shared_memory_limit());
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);

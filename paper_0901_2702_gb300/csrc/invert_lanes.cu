@@ -599,7 +599,8 @@ cudaError_t invert_lanes_slots(int nlam, int64_t npix, int64_t* nslots, int* gri
   constexpr int T = kInvLanes;
   const size_t sm = lanes_smem<T>(nlam);
   cudaError_t e = cudaFuncSetAttribute(invert_lanes_kernel<T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       shared_memory_limit());
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);

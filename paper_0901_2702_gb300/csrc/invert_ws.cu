@@ -684,7 +684,8 @@ template <int NB>
 static cudaError_t ws_slots(int nlam, int64_t npix, int64_t* nslots, int* grid, size_t* smem) {
   auto kern = invert_ws_kernel<6, NB>;
   const size_t sm = WsSmem<NB>(table_floats(6, nlam)).total;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       shared_memory_limit());
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);

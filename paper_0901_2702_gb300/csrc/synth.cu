@@ -262,7 +262,7 @@ static cudaError_t launch_synth_nf(const SynthArgs& a, cudaStream_t s) {
   auto kern = synth_kernel<NF>;
   if (smem > 48 * 1024) {
     cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, shared_memory_limit());
     if (e != cudaSuccess) return e;
   }
   // one CTA per 128 pixels: with a grid of resident CTAs striding over the

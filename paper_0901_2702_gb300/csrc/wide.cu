@@ -907,7 +907,8 @@ cudaError_t launch_wide_synth(const float* params, int64_t npix, const float* ta
                               const LineK& lk, cudaStream_t s) {
   const size_t smem = wide_smem(nf, nlam, false, kWSynthWarps);
   cudaError_t e = cudaFuncSetAttribute(wide_synth_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       shared_memory_limit());
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0, per = 0;
   cudaGetDevice(&dev);
@@ -925,10 +926,10 @@ cudaError_t launch_wide_synth(const float* params, int64_t npix, const float* ta
 }
 
 cudaError_t launch_wide_invert(const InvertArgs& a, int nf, cudaStream_t s) {
-  int dev = 0, nsm = 0, most = 0;
+  int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int most = shared_memory_limit();
   nsm = sm_budget(nsm);
   // one CTA per SM, a pixel a warp: up to 8 warps (65,536 pixels of 112
   // samples 43.0 ms; with 9, what the shared memory holds, 43.3; halving the
@@ -940,9 +941,6 @@ cudaError_t launch_wide_invert(const InvertArgs& a, int nf, cudaStream_t s) {
   if (warps < 1) warps = 1;
   while (warps > 1 && wide_smem(nf, a.nlam, true, (int)warps) > (size_t)most) --warps;
   const size_t smem = wide_smem(nf, a.nlam, true, (int)warps);
-  // the limit belongs to the kernel, not to the call, and the warps, so the
-  // bytes, go by the map: with the call's own bytes as the limit, a thread with
-  // a small map lowered it between another's setting and launch, which then failed
   cudaError_t e = cudaFuncSetAttribute(wide_invert_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
