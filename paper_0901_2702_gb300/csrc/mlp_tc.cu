@@ -50,8 +50,8 @@ constexpr int TM = 128;       // pixels per tile = MMA M
 constexpr int K0 = 32;        // input width (24) padded to two K = 16 steps
 constexpr int N3 = 16;        // output width (11) padded to the smallest N for M = 128
 constexpr int NSLOT = 5;      // weight ring depth
-constexpr int THREADS = 256;  // a group: 4 lane quarters x 2 column halves
-constexpr int kLaunch = 2 * THREADS + 64;  // two groups, a warp that loads weights, one that issues
+constexpr int kCompute = 512;  // 16 warps, in one or two groups, each with a tile in flight
+constexpr int kLaunch = kCompute + 64;  // and a warp that loads weights, one that issues
 constexpr int kPerLayer = HID / 32;  // chunks of a hidden layer
 
 constexpr uint32_t kChunkBytes = HID * 32 * 2;    // 16384
@@ -134,12 +134,17 @@ struct TcArgs {
   int* err;
 };
 
+// G groups: two where a CTA has several tiles; all 16 warps on the one where it
+// has a single tile (up to a tile an SM: 1,000 pixels 32.9 us with one group of
+// eight warps idle, 30.8 so).
+template <int G>
 __global__ void __launch_bounds__(kLaunch, 1) mlp_tc_kernel(TcArgs a) {
+  constexpr int THREADS = kCompute / G;  // a group: 4 lane quarters x 2 or 4 parts of the columns
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t sb = smem_u32(sm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int group = (threadIdx.x / THREADS) & 1, tid = threadIdx.x % THREADS;  // of the group
+  const int group = (threadIdx.x / THREADS) % G, tid = threadIdx.x % THREADS;  // of the group
   float* bias = reinterpret_cast<float*>(sm + SM_BIAS);
   float* stat = reinterpret_cast<float*>(sm + SM_STAT);
   const uint32_t bar_full = sb + SM_BAR, bar_empty = bar_full + 8 * NSLOT,
@@ -184,19 +189,19 @@ __global__ void __launch_bounds__(kLaunch, 1) mlp_tc_kernel(TcArgs a) {
   tc_after_sync();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 2 * THREADS / 32) {
+  if (warp == kCompute / 32) {
     // weight loads: their own warp, so that neither they wait for an issue nor
     // an issue for a slot
     if (lane == 0) {
       Cursor c;
       int loaded = 0;
       bool bad = false;
-      for (int t = 0; t < my_tiles && !bad; t += 2) {
+      for (int t = 0; t < my_tiles && !bad; t += G) {
         const uint8_t* src = a.wp;
         for (int l = 0; l < 4 && !bad; ++l) {
           const int n = layer_chunks(l);
           const uint32_t bytes = l < 3 ? kChunkBytes : kW3Bytes;
-          for (int q = 0; q < (t + 1 < my_tiles ? 2 : 1) && !bad; ++q)
+          for (int q = 0; q < (G == 2 && t + 1 < my_tiles ? 2 : 1) && !bad; ++q)
             for (int i = 0; i < n; ++i, c.next()) {
               // (the first round finds the slots free)
               if (!mbar_wait(bar_empty + 8 * c.slot, c.phase ^ 1)) {
@@ -226,15 +231,15 @@ __global__ void __launch_bounds__(kLaunch, 1) mlp_tc_kernel(TcArgs a) {
     return;
   }
 
-  if (warp == 2 * THREADS / 32 + 1) {
+  if (warp == kCompute / 32 + 1) {
     // the products of both groups, in the order of the stream (every slot's
     // phases are then waited for one after the other)
     if (lane == 0) {
       Cursor c;
       bool bad = false;
-      for (int t = 0; t < my_tiles && !bad; t += 2)
+      for (int t = 0; t < my_tiles && !bad; t += G)
         for (int l = 0; l < 4 && !bad; ++l)
-          for (int q = 0; q < (t + 1 < my_tiles ? 2 : 1) && !bad; ++q) {
+          for (int q = 0; q < (G == 2 && t + 1 < my_tiles ? 2 : 1) && !bad; ++q) {
             // four phases a tile: layer l's has parity l & 1
             if (!mbar_wait(bar_ready + 8 * q, l & 1)) {
               bad = true;
@@ -303,7 +308,7 @@ __global__ void __launch_bounds__(kLaunch, 1) mlp_tc_kernel(TcArgs a) {
   // bias + GELU of the accumulator -> BF16 activations (next layer's A)
   auto epilogue_hidden = [&](const float* b) {
     constexpr int kCols = HID / (THREADS / 128);  // a warp's columns
-    const int q = warp & 3, row = 32 * q + lane, cbeg = ((warp >> 2) & 1) * kCols;
+    const int q = warp & 3, row = 32 * q + lane, cbeg = ((warp >> 2) % (THREADS / 128)) * kCols;
     uint8_t* hrow = H + (row >> 3) * 1024 + (row & 7) * 16;
 #pragma unroll 1
     for (int col0 = cbeg; col0 < cbeg + kCols; col0 += 32) {
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(kLaunch, 1) mlp_tc_kernel(TcArgs a) {
   };
 
   bool ok = true;
-  for (int t = group; t < my_tiles; t += 2) {
+  for (int t = group; t < my_tiles; t += G) {
     const int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
     // features: thread (row, part) writes input columns 8 part .. 8 part + 7
     // and of part + 2
@@ -410,12 +415,13 @@ cudaError_t nn_infer(void* ws, const float* blob, const float* obs, int64_t n, f
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
   nsm = sm_budget(nsm);
-  if ((e = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const int64_t ntiles = (n + TM - 1) / TM;
+  auto kern = ntiles <= nsm ? mlp_tc_kernel<1> : mlp_tc_kernel<2>;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kSmemBytes)) != cudaSuccess)
     return e;
-  const int64_t ntiles = (n + TM - 1) / TM;
   TcArgs a{obs, n, blob, wp, mu, init, conf, raw, static_cast<int*>(ws)};
-  mlp_tc_kernel<<<(unsigned)(ntiles < nsm ? ntiles : nsm), kLaunch, kSmemBytes, s>>>(a);
+  kern<<<(unsigned)(ntiles < nsm ? ntiles : nsm), kLaunch, kSmemBytes, s>>>(a);
   return cudaGetLastError();
 }
 
